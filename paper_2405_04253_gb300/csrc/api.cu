@@ -285,6 +285,10 @@ bool fnt::cdc_use_split(const fnt_plan *p, int64_t n_items) {
     return n_items < 2 * (int64_t)p->n_sm;
 }
 
+// The direct form runs unless a transform kernel was picked (also by
+// arming the transform kernel's test hook).
+bool fnt::cdc_use_direct(const fnt_plan *p) { return p->cdc_kernel == 0 && p->test_inject == 0; }
+
 extern "C" fnt_status fnt_plan_set_test_inject(fnt_plan *p, int32_t mode) {
     if (!p) return fail(FNT_ERR_INVALID, "null plan");
     if (mode != 0 && mode != 1) return fail(FNT_ERR_INVALID, "test inject mode must be 0 or 1");
@@ -325,7 +329,7 @@ bool fnt::aeq_use_serial(const fnt_plan *p, int64_t n_chains, int64_t longest_sy
 }
 
 cudaError_t fnt::aeq_launch_for(const fnt_plan *p, const DevFrame *frames, const AeqChain *chains, int n_chains,
-                                int64_t longest_symbols, cudaStream_t stream) {
+                                int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream) {
     AeqParams prm{p->d.mu_shift, p->d.rde_a, update_period(p->d), p->tensor_gradient, p->d.aeq_freq_sum};
     if (aeq_use_serial(p, n_chains, longest_symbols))
         return aeq_serial_launch(p->d.n_aeq, frames, chains, n_chains, prm, 0, stream);
@@ -439,6 +443,23 @@ static void add_cdc_items(const DevFrame &df, int fi, bool both, std::vector<int
     }
 }
 
+int64_t cdc_direct_tiles(const DevFrame &df, int op) {
+    return ((op == FNT_OP_CHAIN ? df.n_sym : df.n) + kCdcDirectTile - 1) / kCdcDirectTile;
+}
+
+// One-tile items (CTAs of one warp) while that spreads the work over more SMs; above
+// two tiles an SM, four tiles share a CTA and its table entry.
+int cdc_direct_tiles_per_item(const fnt_plan *p, int64_t tiles) {
+    return tiles <= 2 * (int64_t)p->n_sm ? 1 : kCdcDirectWarps;
+}
+
+// Items of the direct CDC for one frame: `per` tiles of all its polarisations each.
+static void add_direct_items(const DevFrame &df, int fi, int op, int per, std::vector<int4> &items) {
+    const int64_t tiles = cdc_direct_tiles(df, op);
+    for (int64_t t = 0; t < tiles; t += per)
+        items.push_back(make_int4(fi, (int)t, (int)std::min<int64_t>(per, tiles - t), 0));
+}
+
 // Whether the CDC items of this work take both polarisations at once.  Per-
 // polarisation items double the warps (better for work that does not fill the
 // GPU twice over); two-polarisation items halve the window fills and the tap
@@ -516,12 +537,21 @@ fnt_status build_work(const fnt_plan *p, const fnt_frame_batch *b, int op, Work 
     if (op == FNT_OP_CHAIN)
         std::stable_sort(order.begin(), order.end(),
                          [&](int a, int c) { return w.frames[a].n_sym > w.frames[c].n_sym; });
-    const bool both = op != FNT_OP_AEQ && cdc_items_both(p, w);
+    w.cdc_direct = op != FNT_OP_AEQ && cdc_use_direct(p);
+    const bool both = op != FNT_OP_AEQ && !w.cdc_direct && cdc_items_both(p, w);
     w.cdc_both = both;
+    if (w.cdc_direct) {
+        int64_t tiles = 0;
+        for (const DevFrame &df : w.frames) tiles += cdc_direct_tiles(df, op);
+        w.cdc_tiles = cdc_direct_tiles_per_item(p, tiles);
+    }
     {
         size_t n_items = 0, n_chains = 0;
         for (const DevFrame &df : w.frames) {
-            if (op != FNT_OP_AEQ) n_items += (size_t)(((df.n + df.S - 1) / df.S + kBlocksPerItem - 1) / kBlocksPerItem) * 2;
+            if (w.cdc_direct)
+                n_items += (size_t)((cdc_direct_tiles(df, op) + w.cdc_tiles - 1) / w.cdc_tiles);
+            else if (op != FNT_OP_AEQ)
+                n_items += (size_t)(((df.n + df.S - 1) / df.S + kBlocksPerItem - 1) / kBlocksPerItem) * 2;
             if (op != FNT_OP_CDC)
                 n_chains += p->d.aeq_segment > 0 ? (size_t)((df.n_sym + p->d.aeq_segment - 1) / p->d.aeq_segment) : 1;
         }
@@ -530,13 +560,21 @@ fnt_status build_work(const fnt_plan *p, const fnt_frame_batch *b, int op, Work 
     }
     for (int i : order) {
         const int first_item = (int)w.items.size();
-        if (op != FNT_OP_AEQ) add_cdc_items(w.frames[i], i, both, w.items);
+        if (w.cdc_direct)
+            add_direct_items(w.frames[i], i, op, w.cdc_tiles, w.items);
+        else if (op != FNT_OP_AEQ)
+            add_cdc_items(w.frames[i], i, both, w.items);
         if (op != FNT_OP_CDC) {
             const size_t c0 = w.chains.size();
             add_aeq_chains(p, w.frames[i], i, p->d_init, w);
             for (size_t c = c0; c < w.chains.size(); ++c) {
                 const DevFrame &df = w.frames[i];
-                // last 2-sps sample the chain reads, and the CDC item that produces it
+                // the CDC item that produces the last symbol the chain reads (transform
+                // items: the last 2-sps sample's)
+                if (w.cdc_direct) {
+                    w.chains[c].need_item = first_item + (int)((w.chains[c].end - 1) / kCdcDirectTile / w.cdc_tiles);
+                    continue;
+                }
                 const int64_t t_last = 2 * (w.chains[c].end - 1) + df.phase;
                 const int per = both && df.n_pol == 2 ? 1 : df.n_pol;     // items per 32 blocks
                 w.chains[c].need_item =
@@ -583,7 +621,7 @@ void layout(Work &w) {
     w.off_chains = up(w.off_items + w.items.size() * sizeof(int4));
     w.off_init = up(w.off_chains + w.chains.size() * sizeof(AeqChain));
     w.off_spec = up(w.off_init + w.init_src.size() * kStateBytes);
-    w.off_scratch = up(w.off_spec + (w.op != FNT_OP_AEQ ? w.frames.size() * kSpecBytes : 0));
+    w.off_scratch = up(w.off_spec + (w.op != FNT_OP_AEQ && !w.cdc_direct ? w.frames.size() * kSpecBytes : 0));
     w.total = up(w.off_scratch + (size_t)w.scratch_bytes);
     if (w.total == 0) w.total = 256;
 }
@@ -634,7 +672,7 @@ static Staging &thread_staging() {
 }
 
 void point_spectra(Work &w, char *dev) {
-    if (w.op == FNT_OP_AEQ) return;
+    if (w.op == FNT_OP_AEQ || w.cdc_direct) return;
     for (size_t i = 0; i < w.frames.size(); ++i)
         w.frames[i].hspec = (int32_t *)(dev + w.off_spec + i * kSpecBytes);
 }
@@ -667,6 +705,11 @@ static fnt_status launch_cdc_range(const fnt_plan *p, const Work &w, const char 
                                    cudaStream_t stream) {
     if (i1 <= i0) return FNT_OK;
     const DevFrame *frames = (const DevFrame *)(dev + w.off_frames);
+    if (w.cdc_direct) {
+        cudaError_t e = cdc_direct_launch(frames, (const int4 *)(dev + w.off_items) + i0, i1 - i0,
+                                          w.op == FNT_OP_CHAIN, w.cdc_tiles, stream);
+        return e == cudaSuccess ? FNT_OK : cuda_fail(e, "direct cdc kernel launch");
+    }
     const int nw = p->cdc_warps;
     const int n = i1 - i0;
     const int grid = std::min((n + nw - 1) / nw, p->n_sm * 64);
@@ -688,14 +731,18 @@ static fnt_status launch_aeq_range(const fnt_plan *p, const Work &w, const char 
                                    cudaStream_t stream) {
     if (c1 <= c0) return FNT_OK;
     const DevFrame *frames = (const DevFrame *)(dev + w.off_frames);
-    int64_t longest = 0;                  // chains are sorted longest first within a chunk; take the max anyway
-    for (int c = c0; c < c1; ++c) longest = std::max(longest, w.chains[c].end - w.chains[c].begin);
-    cudaError_t e = aeq_launch_for(p, frames, (const AeqChain *)(dev + w.off_chains) + c0, c1 - c0, longest, stream);
+    int64_t longest = 0, total = 0;       // chains are sorted longest first within a chunk; take the max anyway
+    for (int c = c0; c < c1; ++c) {
+        longest = std::max(longest, w.chains[c].end - w.chains[c].begin);
+        total += w.chains[c].end - w.chains[c].begin;
+    }
+    cudaError_t e = aeq_launch_for(p, frames, (const AeqChain *)(dev + w.off_chains) + c0, c1 - c0, total, longest,
+                                   stream);
     return e == cudaSuccess ? FNT_OK : cuda_fail(e, "aeq kernel launch");
 }
 
 static fnt_status launch_spectra(const Work &w, const char *dev, cudaStream_t stream) {
-    if (w.op == FNT_OP_AEQ || w.spectra_ready || w.frames.empty()) return FNT_OK;
+    if (w.op == FNT_OP_AEQ || w.cdc_direct || w.spectra_ready || w.frames.empty()) return FNT_OK;
     cudaError_t e = cdc_spectra_launch((const DevFrame *)(dev + w.off_frames), (int)w.frames.size(), stream);
     return e == cudaSuccess ? FNT_OK : cuda_fail(e, "tap spectra launch");
 }
@@ -740,7 +787,7 @@ fnt_status launch_pipelined(const fnt_plan *p, const Work &w, const char *dev, c
 int work_kernel_count(const Work &w) {
     const int C = (int)w.item_cut.size() - 1;
     int k = 0;
-    if (w.op != FNT_OP_AEQ && !w.spectra_ready && !w.frames.empty()) k += 1;   // tap spectra
+    if (w.op != FNT_OP_AEQ && !w.cdc_direct && !w.spectra_ready && !w.frames.empty()) k += 1;   // tap spectra
     if (w.op != FNT_OP_AEQ) k += C > 1 ? C : (w.items.empty() ? 0 : 1);
     if (w.op != FNT_OP_CDC) {
         if (C > 1) {

@@ -53,6 +53,8 @@ int64_t chain_nsym(int64_t n, int phase);
 struct Work {
     int op = 0;
     bool cdc_both = false;            // CDC items may cover both polarisations (item.w = 2)
+    bool cdc_direct = false;          // CDC items are the direct kernel's (tiles of a frame)
+    int cdc_tiles = 1;                // direct CDC: most tiles per item
     bool spectra_ready = false;       // the frames' CDC tap spectra are computed (prepared batches)
     std::vector<DevFrame> frames;
     std::vector<int4> items;          // CDC: (frame, first block, blocks)
@@ -91,6 +93,8 @@ int work_kernel_count(const Work &w);
 constexpr int kCdcCtasPerSm = 3;     // cdc_kernel's __launch_bounds__ minimum
 constexpr int kSerialCtasPerSm = 1;  // aeq_serial_kernel CTAs resident per SM (registers)
 constexpr int kSerialMinBlocks = 256;  // shortest longest-chain (blocks) for which the automatic choice takes it
+cudaError_t cdc_direct_launch(const DevFrame *frames, const int4 *items, int n_items, bool chain, int warps,
+                              cudaStream_t stream);
 size_t cdc_smem_bytes(int warps);
 int cdc_mults_per_block();
 int cdc_butterflies_per_block();
@@ -116,8 +120,13 @@ cudaError_t aeq_serial_launch(int na, const DevFrame *frames, const AeqChain *ch
 // Whether a launch of n_chains chains, the longest of longest_symbols symbols,
 // takes the CTA-per-chain kernel.
 bool aeq_use_serial(const fnt_plan *p, int64_t n_chains, int64_t longest_symbols);
-// Launches the AEQ kernel the plan picks for those chains.
+// Launches the AEQ kernel the plan picks for those chains, of total_symbols in all.
 cudaError_t aeq_launch_for(const fnt_plan *p, const DevFrame *frames, const AeqChain *chains, int n_chains,
-                           int64_t longest_symbols, cudaStream_t stream);
+                           int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream);
+// Whether the plan's CDC runs in direct form (no transform kernel picked).
+bool cdc_use_direct(const fnt_plan *p);
+// Tiles of a frame's direct CDC for `op`, and how many of `tiles` an item takes.
+int64_t cdc_direct_tiles(const DevFrame &df, int op);
+int cdc_direct_tiles_per_item(const fnt_plan *p, int64_t tiles);
 
 }  // namespace fnt

@@ -13,6 +13,11 @@ constexpr int kBlocksPerItem = 32; // CDC blocks per warp work item (one per lan
 // CDC work item: int4 (frame, first block, blocks, polarisation); a group of 32
 // blocks of an n_pol = 2 frame is two consecutive items (pol 0, pol 1).
 
+// The direct CDC kernel's work item: int4 (frame, first tile, tiles, 0), a tile being
+// the outputs of a warp (CDC: samples, chain: symbols) in all polarisations.
+constexpr int kCdcDirectTile = 256;
+constexpr int kCdcDirectWarps = 4;   // most tiles per item (a warp each)
+
 // One frame as the kernels see it (16-byte aligned).
 struct alignas(16) DevFrame {
     const int8_t *in;      // CDC / chain: int8 [n][n_pol][2]; AEQ alone: int8 [n][4]

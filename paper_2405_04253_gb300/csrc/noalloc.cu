@@ -168,11 +168,19 @@ extern "C" fnt_status fnt_cdc_aeq_run_noalloc(const fnt_plan *p, const fnt_frame
     memcpy(df.taps, f->cd_taps, 2 * (size_t)f->cd_len);
 
     int4 *items = (int4 *)(mir + kOffItems);
-    const int64_t nblk = (f->n + S - 1) / S;
     int n_items = 0;
-    for (int64_t b = 0; b < nblk; b += kBlocksPerItem)
-        for (int pol = 0; pol < 2; ++pol)
-            items[n_items++] = make_int4(0, (int)b, (int)std::min<int64_t>(kBlocksPerItem, nblk - b), pol);
+    const bool direct = cdc_use_direct(p);
+    const int64_t tiles = cdc_direct_tiles(df, FNT_OP_CHAIN);
+    const int per = cdc_direct_tiles_per_item(p, tiles);   // n / 512 tiles at most: fits kMaxItems
+    if (direct) {
+        for (int64_t t = 0; t < tiles; t += per)
+            items[n_items++] = make_int4(0, (int)t, (int)std::min<int64_t>(per, tiles - t), 0);
+    } else {
+        const int64_t nblk = (f->n + S - 1) / S;
+        for (int64_t b = 0; b < nblk; b += kBlocksPerItem)
+            for (int pol = 0; pol < 2; ++pol)
+                items[n_items++] = make_int4(0, (int)b, (int)std::min<int64_t>(kBlocksPerItem, nblk - b), pol);
+    }
 
     // the chains follow the items (kOffChains bounds them for the largest frame)
     const size_t off_chains = (kOffItems + (size_t)n_items * sizeof(int4) + 255) / 256 * 256;
@@ -208,19 +216,26 @@ extern "C" fnt_status fnt_cdc_aeq_run_noalloc(const fnt_plan *p, const fnt_frame
 
     const DevFrame *frames = (const DevFrame *)(base + kOffFrame);
     const int nw = p->cdc_warps;
-    e = cdc_spectra_launch(frames, 1, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "noalloc: tap spectra launch");
-    e = cdc_launch(frames, (const int4 *)(base + kOffItems), n_items, true, false, nw,
-                   std::min((n_items + nw - 1) / nw, p->n_sm * 64), stream, cdc_use_split(p, n_items));
+    if (direct) {
+        e = cdc_direct_launch(frames, (const int4 *)(base + kOffItems), n_items, true, per, stream);
+    } else {
+        e = cdc_spectra_launch(frames, 1, stream);
+        if (e != cudaSuccess) return cuda_fail(e, "noalloc: tap spectra launch");
+        e = cdc_launch(frames, (const int4 *)(base + kOffItems), n_items, true, false, nw,
+                       std::min((n_items + nw - 1) / nw, p->n_sm * 64), stream, cdc_use_split(p, n_items));
+    }
     if (e != cudaSuccess) return cuda_fail(e, "noalloc: cdc kernel launch");
     if (nc > 0) {
         if (n_chains > 1 && f->aeq_state) {
             e = cudaMemcpyAsync(base + kOffInit, f->aeq_state, kStateBytes, cudaMemcpyDeviceToDevice, stream);
             if (e != cudaSuccess) return cuda_fail(e, "noalloc: copy initial taps");
         }
-        int64_t longest = 0;
-        for (int c = 0; c < nc; ++c) longest = std::max(longest, chains[c].end - chains[c].begin);
-        e = aeq_launch_for(p, frames, (const AeqChain *)(base + off_chains), nc, longest, stream);
+        int64_t longest = 0, total = 0;
+        for (int c = 0; c < nc; ++c) {
+            longest = std::max(longest, chains[c].end - chains[c].begin);
+            total += chains[c].end - chains[c].begin;
+        }
+        e = aeq_launch_for(p, frames, (const AeqChain *)(base + off_chains), nc, total, longest, stream);
         if (e != cudaSuccess) return cuda_fail(e, "noalloc: aeq kernel launch");
     }
     return FNT_OK;

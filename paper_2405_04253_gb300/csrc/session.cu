@@ -221,6 +221,12 @@ fnt_status launch_wave(fnt_session *ss, cudaStream_t stream, Wave &wave, cudaEve
     w.op = FNT_OP_CHAIN;
     const int nf = (int)wave.reqs.size();
     w.frames.resize(nf);
+    w.cdc_direct = cdc_use_direct(ss->plan);
+    if (w.cdc_direct) {
+        int64_t tiles = 0;
+        for (const Request &r : wave.reqs) tiles += (r.n_sym + kCdcDirectTile - 1) / kCdcDirectTile;
+        w.cdc_tiles = cdc_direct_tiles_per_item(ss->plan, tiles);
+    }
     for (int i = 0; i < nf; ++i) {
         const Request &r = wave.reqs[i];
         const LinkState &lk = ss->links[r.link];
@@ -238,10 +244,16 @@ fnt_status launch_wave(fnt_session *ss, cudaStream_t stream, Wave &wave, cudaEve
         df.shift = lk.shift;
         df.phase = lk.phase;
         memcpy(df.taps, lk.taps, sizeof df.taps);
-        const int64_t nblk = (r.n + lk.S - 1) / lk.S;
-        for (int64_t b = 0; b < nblk; b += kBlocksPerItem)
-            for (int pol = 0; pol < 2; ++pol)
-                w.items.push_back(make_int4(i, (int)b, (int)std::min<int64_t>(kBlocksPerItem, nblk - b), pol));
+        if (w.cdc_direct) {
+            const int64_t tiles = cdc_direct_tiles(df, FNT_OP_CHAIN);
+            for (int64_t t = 0; t < tiles; t += w.cdc_tiles)
+                w.items.push_back(make_int4(i, (int)t, (int)std::min<int64_t>(w.cdc_tiles, tiles - t), 0));
+        } else {
+            const int64_t nblk = (r.n + lk.S - 1) / lk.S;
+            for (int64_t b = 0; b < nblk; b += kBlocksPerItem)
+                for (int pol = 0; pol < 2; ++pol)
+                    w.items.push_back(make_int4(i, (int)b, (int)std::min<int64_t>(kBlocksPerItem, nblk - b), pol));
+        }
         if (r.n_sym > 0 && !segmented(ss->plan, r.n_sym)) {
             AeqChain c{};
             c.frame = i;
