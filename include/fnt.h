@@ -143,7 +143,7 @@ FNT_API fnt_status fnt_plan_create(const fnt_plan_desc *desc, fnt_plan **out);
 /* Waits for the device, then frees the plan and its memory pool. */
 FNT_API fnt_status fnt_plan_destroy(fnt_plan *plan);
 
-/* Multiplication counts of the kernels for a plan description (no device
+/* Multiplication counts of the transform kernels for a plan description (no device
  * needed), in the units of Tab. 1
  * (real multiplications per symbol; twiddle products by powers of the radix
  * are not counted, as in the paper, since they are shifts in its hardware).
@@ -310,32 +310,37 @@ FNT_API fnt_status fnt_plan_set_pipeline(fnt_plan *plan, int32_t chunks);
 /* Caps the AEQ warps resident per SM for later launches of this plan
  * (autotuner hook): each AEQ CTA then reserves enough shared memory that at
  * most max(1, max_warps_per_sm / aeq warps per CTA) CTAs share an SM.  0
- * (default) lets resources decide.  Long serial AEQ chains (frames with fresh
+ * (default) lets resources decide (transform kernels only, see
+ * fnt_plan_set_aeq_kernel).  Long serial AEQ chains (frames with fresh
  * taps and no segments) finish sooner when fewer share an SM, which can
  * shorten a batch whose longest chain sets its time.  Results do not depend on
  * it.  FNT_ERR_INVALID outside [0, 64]. */
 FNT_API fnt_status fnt_plan_set_aeq_occupancy(fnt_plan *plan, int32_t max_warps_per_sm);
 
-/* Picks the AEQ kernel of later launches of this plan: 1 = one warp per (chain,
- * polarisation), the throughput layout for many chains; 2 = one CTA per (chain,
- * polarisation), which spreads each block of the serial recurrence of eq. (6)
- * (section "Proposed FNT-CDC&AEQ structure") over 288 threads and cuts the time
- * per block of a lone chain; 0 (default) = 2 when the launch's chains fit one
- * CTA per SM and its longest chain has at least 256 AEQ blocks, else 1 (short
- * chains, such as the segments of served frames, do better in 1 when several
- * launches share the GPU, as each CTA of 2 holds a whole SM).  Plans with
- * aeq_freq_sum != 0 always use 1.  Results do not depend on it.
+/* Picks the AEQ kernel of later launches of this plan.  0 (default): the direct
+ * form, whose convolutions and gradient are exact integer dot products (constraint
+ * (5) makes the transforms' convolutions the same integers), except that plans with
+ * aeq_freq_sum = 1, whose sums wrap in Z_F, run as with 1.  1 and 2 run the Fermat
+ * number transforms: 1 = one warp per (chain, polarisation), the throughput layout
+ * for many chains; 2 = one CTA per (chain, polarisation), which spreads each block
+ * of the serial recurrence of eq. (6) (section "Proposed FNT-CDC&AEQ structure")
+ * over 288 threads and cuts the time per block of a lone chain.  Plans with
+ * aeq_freq_sum != 0 run 1 where 2 is asked for.  Results do not depend on it for
+ * samples and taps inside the ranges stated above.  The warps per CTA, the occupancy
+ * cap and the tensor-core gradient set on a plan apply to kernels 1 and 2.
  * FNT_ERR_INVALID outside [0, 2]. */
 FNT_API fnt_status fnt_plan_set_aeq_kernel(fnt_plan *plan, int32_t kind);
 
-/* Picks the CDC kernel of later launches of this plan: 1 = one overlap-save
- * block per lane (each 64-point transform in one thread's registers), the
- * throughput layout; 2 = one block per 8 threads, each transform run as a
- * four-step 8 x 8 transform over them (eqs. (1)/(2) split by index, section
+/* Picks the CDC kernel of the calls and prepared batches made later with this plan.
+ * 0 (default): the direct form (exact integer dot products; constraint (5) makes
+ * the transforms' convolution the same integers).  1 and 2 run the 64-point
+ * transforms: 1 = one overlap-save block per lane (each transform in one thread's
+ * registers), the throughput layout; 2 = one block per 8 threads, each transform
+ * run as a four-step 8 x 8 transform over them (eqs. (1)/(2) split by index, section
  * "Fermat number transform"), for work too small to fill the GPU one block per
- * lane; 0 (default) = 2 when a launch has fewer 32-block work items than twice
- * the SM count, else 1.  Results do not depend on it.  FNT_ERR_INVALID
- * outside [0, 2]. */
+ * lane.  Results do not depend on it for samples and taps inside the ranges stated
+ * above.  The warps per CTA and polarisations per item set on a plan apply to
+ * kernels 1 and 2.  FNT_ERR_INVALID outside [0, 2]. */
 FNT_API fnt_status fnt_plan_set_cdc_kernel(fnt_plan *plan, int32_t kind);
 
 /* The one-block-per-lane CDC kernel fetches the 32 input windows of a PDM work
@@ -361,14 +366,18 @@ FNT_API fnt_status fnt_device_faults(int32_t clear, uint32_t *faults);
  * FNT_ERR_INVALID for other modes. */
 FNT_API fnt_status fnt_plan_set_test_inject(fnt_plan *plan, int32_t mode);
 
-/* The CDC kernel (1 or 2, as above) a launch of `n_items` CDC work items (32
- * overlap-save blocks of one polarisation, or of both) of this plan takes; 0
- * for a null plan. */
+/* The transform CDC kernel (1 or 2, as above) for a launch of `n_items` CDC work
+ * items (32 overlap-save blocks of one polarisation, or of both): the one picked on
+ * the plan, else 2 below twice the SM count and 1 from there on.  A plan that picks
+ * none runs the direct form instead.  0 for a null plan. */
 FNT_API int32_t fnt_plan_cdc_kernel_for(const fnt_plan *plan, int64_t n_items);
 
-/* The AEQ kernel (1 or 2, as above) a launch of `n_chains` AEQ chains of this
- * plan, the longest of `longest_symbols` symbols, takes; 0 for a null plan.
- * A chain is a frame, or one AEQ segment of a frame with its warm-up. */
+/* The transform AEQ kernel (1 or 2, as above) for a launch of `n_chains` AEQ chains,
+ * the longest of `longest_symbols` symbols: the one picked on the plan, else 2 when
+ * the chains fit one CTA per SM and the longest has at least 256 AEQ blocks, else 1.
+ * A plan that picks none runs the direct form instead (aeq_freq_sum = 1: kernel 1).
+ * A chain is a frame, or one AEQ segment of a frame with its warm-up.  0 for a null
+ * plan. */
 FNT_API int32_t fnt_plan_aeq_kernel_for(const fnt_plan *plan, int64_t n_chains, int64_t longest_symbols);
 
 /* The plan's initial AEQ taps (the state a frame without aeq_state, or a newly

@@ -221,13 +221,13 @@ class Plan:
         check(lib().fnt_plan_set_aeq_occupancy(self.handle, int(max_warps_per_sm)))
 
     def set_aeq_kernel(self, kind: int):
-        """AEQ kernel: 1 a warp per (chain, polarisation), 2 a CTA per one,
-        0 automatic; same results."""
+        """AEQ kernel: 0 the direct form (exact integer dot products), 1 and 2 the
+        transforms, a warp (1) or a CTA (2) per (chain, polarisation); same results."""
         check(lib().fnt_plan_set_aeq_kernel(self.handle, int(kind)))
 
     def set_cdc_kernel(self, kind: int):
-        """CDC kernel: 1 a block per lane, 2 a block per 8 threads, 0
-        automatic; same results."""
+        """CDC kernel: 0 the direct form (exact integer dot products), 1 and 2 the
+        transforms, a block per lane (1) or per 8 threads (2); same results."""
         check(lib().fnt_plan_set_cdc_kernel(self.handle, int(kind)))
 
     def set_test_inject(self, mode: int):
@@ -236,12 +236,12 @@ class Plan:
         check(lib().fnt_plan_set_test_inject(self.handle, int(mode)))
 
     def cdc_kernel_for(self, n_items: int) -> int:
-        """The CDC kernel (1 or 2) a launch of n_items 32-block work items takes."""
+        """The transform CDC kernel (1 or 2) for a launch of n_items 32-block work items."""
         return int(lib().fnt_plan_cdc_kernel_for(self.handle, int(n_items)))
 
     def aeq_kernel_for(self, n_chains: int, longest_symbols: int) -> int:
-        """The AEQ kernel (1 or 2) a launch of n_chains chains, the longest of
-        longest_symbols symbols, takes."""
+        """The transform AEQ kernel (1 or 2) for a launch of n_chains chains, the
+        longest of longest_symbols symbols."""
         return int(lib().fnt_plan_aeq_kernel_for(self.handle, int(n_chains), int(longest_symbols)))
 
     def initial_state(self) -> np.ndarray:

@@ -13,7 +13,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libfnt.so")
 
-SOURCES = ["cdc_direct.cu", "cdc.cu", "aeq.cu", "aeq_serial.cu", "api.cu", "session.cu", "noalloc.cu"]
+SOURCES = ["cdc_direct.cu", "aeq_direct.cu", "cdc.cu", "aeq.cu", "aeq_serial.cu", "api.cu", "session.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC",
          "-Xcompiler", "-fvisibility=hidden", "-I", INCLUDE, "-I", CSRC]

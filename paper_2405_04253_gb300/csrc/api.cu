@@ -285,9 +285,12 @@ bool fnt::cdc_use_split(const fnt_plan *p, int64_t n_items) {
     return n_items < 2 * (int64_t)p->n_sm;
 }
 
-// The direct form runs unless a transform kernel was picked (also by
-// arming the transform kernel's test hook).
+// The direct forms run unless a transform kernel was picked (for the CDC, also by
+// arming the transform kernel's test hook).  Sums in Z_F that wrap (aeq_freq_sum 1)
+// are defined by the transforms and stay with them.
 bool fnt::cdc_use_direct(const fnt_plan *p) { return p->cdc_kernel == 0 && p->test_inject == 0; }
+
+bool fnt::aeq_use_direct(const fnt_plan *p) { return p->aeq_kernel == 0 && p->d.aeq_freq_sum != 1; }
 
 extern "C" fnt_status fnt_plan_set_test_inject(fnt_plan *p, int32_t mode) {
     if (!p) return fail(FNT_ERR_INVALID, "null plan");
@@ -331,6 +334,9 @@ bool fnt::aeq_use_serial(const fnt_plan *p, int64_t n_chains, int64_t longest_sy
 cudaError_t fnt::aeq_launch_for(const fnt_plan *p, const DevFrame *frames, const AeqChain *chains, int n_chains,
                                 int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream) {
     AeqParams prm{p->d.mu_shift, p->d.rde_a, update_period(p->d), p->tensor_gradient, p->d.aeq_freq_sum};
+    if (aeq_use_direct(p))
+        return aeq_direct_launch(p->d.n_aeq, frames, chains, n_chains, total_symbols, longest_symbols, prm, p->n_sm,
+                                 stream);
     if (aeq_use_serial(p, n_chains, longest_symbols))
         return aeq_serial_launch(p->d.n_aeq, frames, chains, n_chains, prm, 0, stream);
     return aeq_launch(p->d.n_aeq, frames, chains, n_chains, prm, p->aeq_warps, 0, stream, aeq_min_smem(p));

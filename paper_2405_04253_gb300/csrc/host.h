@@ -123,8 +123,13 @@ bool aeq_use_serial(const fnt_plan *p, int64_t n_chains, int64_t longest_symbols
 // Launches the AEQ kernel the plan picks for those chains, of total_symbols in all.
 cudaError_t aeq_launch_for(const fnt_plan *p, const DevFrame *frames, const AeqChain *chains, int n_chains,
                            int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream);
-// Whether the plan's CDC runs in direct form (no transform kernel picked).
+// The direct form of the AEQ (aeq_direct.cu).
+cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
+                              int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
+                              cudaStream_t stream);
+// Whether the plan's CDC and AEQ run in direct form (no transform kernel picked).
 bool cdc_use_direct(const fnt_plan *p);
+bool aeq_use_direct(const fnt_plan *p);
 // Tiles of a frame's direct CDC for `op`, and how many of `tiles` an item takes.
 int64_t cdc_direct_tiles(const DevFrame &df, int op);
 int cdc_direct_tiles_per_item(const fnt_plan *p, int64_t tiles);
