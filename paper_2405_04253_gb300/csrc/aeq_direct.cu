@@ -12,19 +12,14 @@
 // Results are the same integers for every input inside the documented ranges
 // (5-bit symbols, 14-bit taps).
 //
-// One item is a (chain, polarisation): the outputs 2p and 2p + 1 of one run, whose
-// blocks of SA = N - 16 symbols follow each other through the tap update.  A warp
-// holds lane = 16 o + i: first output o, symbol i of 16 (convolution, RDE error),
-// then output o, tap k = i of all four inputs (gradient, update), so a block of 16
-// symbols needs no reduction over lanes and two __syncwarp.
-//   convolution  y_o[i] = sum_s1,k W_o,s1[k] x_s1[t0 + i - k]: four 16-byte loads of
-//                symbol bytes, eight of taps, 32 dp2a
+// Per block of SA = N - 16 symbols and output:
+//   convolution  y_o[i] = sum_s1,k W_o,s1[k] x_s1[t0 + i - k]
 //   error        z = sat16(y >> 7), one shuffle for the other output, e in 32 bits
 //   gradient     G = sum_i e z_o[i] x_s1[t0 + i - k] with e z = c1 2^16 + c0
 //                (c0 16 bits, c1 signed 16 bits) and, only when some |e z| of the
-//                warp's symbols reaches 2^31, c2 2^32: two (three) dp2a for two
-//                products; limb sums are exact in 32 bits, then combined in 64
-//   update       eq. (6) on the lane's own four master taps
+//                block reaches 2^31, c2 2^32: two (three) dp2a for two products;
+//                limb sums are exact in 32 bits, then combined in 64
+//   update       eq. (6) on the master taps, published as 16-bit taps
 //
 // Staged symbols.  xq[q] holds, for the four inputs, the four bytes of symbols
 // q .. q + 3 (a 4 x 4 byte transpose at every q, 16 bytes a symbol), so both the
@@ -32,15 +27,11 @@
 // symbols of an input) read aligned 16-byte words at any offset.  A batch of
 // blocks is transposed at once while the next batch's words arrive by cp.async.
 //
-// Layouts <SYM, GRP, Q>: SA = 16 SYM GRP symbols, GRP Q warps per item.
-//   SYM  symbol groups of 16 a warp works through (3 x 16 at N = 64)
-//   GRP  warps that share a block by symbols.  Each keeps a copy of the taps, forms
-//        the gradient of its own 16 symbols, and the partial sums cross once per
-//        update through shared memory: one barrier a block.
-//   Q    warps that share the gradient and the update by input s1; each repeats the
-//        convolution (its pipes would idle).  One barrier a block, taps double
-//        buffered.
-// aeq_direct_launch picks the layout (rule and figures there).
+// Two layouts; aeq_direct_launch picks one (rule and figures there).
+//   aeq_pair_kernel   a warp per chain, both polarisations: many chains, bound by
+//                     dp2a issue and shared-memory loads
+//   aeq_split_kernel  five warps per (chain, polarisation): few chains, bound by the
+//                     latency of one block
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -52,21 +43,15 @@ namespace fnt {
 
 namespace {
 
-template <int SYM_, int GRP_, int Q_>
+template <int NA>
 struct DirCfg {
     static constexpr int K = kAeqK;
-    static constexpr int SYM = SYM_, GRP = GRP_, Q = Q_;
-    static constexpr int SA = 16 * SYM * GRP;             // symbols per block
-    static constexpr int W = GRP * Q;                     // warps per item
-    static constexpr int NT = 32 * W;
-    static constexpr int NS = 4 / Q;                      // inputs s1 whose gradient a lane holds
-    static constexpr int PB = SA == 48 ? 4 : 8;           // blocks per staged batch
+    static constexpr int SA = NA - K;                     // symbols per block
+    static constexpr int NG = SA / 4;                     // groups of four symbols
+    static constexpr int PB = NA == 64 ? 4 : 8;           // blocks per staged batch
     static constexpr int B = PB * SA;                     // symbols per staged batch
     static constexpr int XW = K + B;                      // staged words: K of history
-    static constexpr int WO = 36;                         // words per output in a tap set (bank shift 4)
-    static constexpr int WS = 2 * WO;                     // words per tap set
-    static constexpr int NG = 4 * SYM * GRP;              // groups of four symbols
-    static_assert(K == 16 && (GRP == 1 || Q == 1) && 4 % Q == 0, "layouts");
+    static_assert(K == 16 && SA % 16 == 0, "shapes");
 };
 
 template <bool AS, bool HI>
@@ -97,12 +82,9 @@ __device__ __forceinline__ void cp_async4(uint32_t *smem, const uint32_t *gmem, 
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-template <int W>
-__device__ __forceinline__ void item_sync() {
-    if constexpr (W == 1)
-        __syncwarp();
-    else
-        __syncthreads();
+template <int ID, int N>
+__device__ __forceinline__ void bar_sync() {
+    asm volatile("bar.sync %0, %1;\n" ::"n"(ID), "n"(N) : "memory");
 }
 
 // clamp(T + d, 30-bit master tap range): the sum saturated to 32 bits, then clamped
@@ -113,248 +95,437 @@ __device__ __forceinline__ int32_t add_tap(int32_t T, int64_t d) {
     return min(max(w, -(1 << 29)), (1 << 29) - 1);
 }
 
-// xn: staged words of symbols tb - K + q, q < XW; xq: their byte transposes.
+// A warp's copies of symbols tb - K + q, q < XW (zero outside [lo, end)), to xn.
 template <class C>
 __device__ __forceinline__ void stage(uint32_t *xn, const uint32_t *xin, int64_t tb, int64_t lo, int64_t end,
-                                      int tid) {
-    for (int q = tid; q < C::XW; q += C::NT) {
-        const int64_t t = tb - C::K + q;
-        const bool ok = t >= lo && t < end;
-        cp_async4(xn + q, ok ? xin + t : xin, ok);
+                                      int lane) {
+    const int64_t t0 = tb - C::K;
+    const uint32_t *src = xin + t0;
+    // positions with t inside [lo, end)
+    const int q0 = (int)min(max(lo - t0, (int64_t)0), (int64_t)C::XW);
+    const int q1 = (int)min(max(end - t0, (int64_t)0), (int64_t)C::XW);
+#pragma unroll
+    for (int q = lane; q < (C::XW + 31) / 32 * 32; q += 32) {
+        if (q >= C::XW) break;
+        const bool ok = q >= q0 && q < q1;
+        cp_async4(xn + q, ok ? src + q : xin, ok);
     }
 }
 
+// xq[q] <- the byte transpose of the staged words q .. q + 3, by one warp, four
+// words of q a lane at a time (loads before stores).
 template <class C>
-__device__ __forceinline__ void transpose(const uint32_t *xn, uint4 *xq, int tid) {
-    for (int q = tid; q < C::XW - 3; q += C::NT) {
-        const uint32_t a = xn[q], b = xn[q + 1], c = xn[q + 2], d = xn[q + 3];
-        const uint32_t ab0 = __byte_perm(a, b, 0x5140), ab1 = __byte_perm(a, b, 0x7362);   // (a0 b0 a1 b1), (a2 b2 a3 b3)
-        const uint32_t cd0 = __byte_perm(c, d, 0x5140), cd1 = __byte_perm(c, d, 0x7362);
-        xq[q] = make_uint4(__byte_perm(ab0, cd0, 0x5410), __byte_perm(ab0, cd0, 0x7632),
-                           __byte_perm(ab1, cd1, 0x5410), __byte_perm(ab1, cd1, 0x7632));
+__device__ __forceinline__ void transpose(const uint32_t *xn, uint4 *xq, int lane) {
+    constexpr int NQ = C::XW - 3;
+#pragma unroll
+    for (int q0 = 0; q0 < NQ; q0 += 128) {
+        uint32_t w[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) w[j][c] = q0 + 32 * j < NQ ? xn[min(q0 + 32 * j + lane, NQ - 1) + c] : 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int q = q0 + 32 * j + lane;
+            const uint32_t ab0 = __byte_perm(w[j][0], w[j][1], 0x5140), ab1 = __byte_perm(w[j][0], w[j][1], 0x7362);
+            const uint32_t cd0 = __byte_perm(w[j][2], w[j][3], 0x5140), cd1 = __byte_perm(w[j][2], w[j][3], 0x7362);
+            if (q0 + 32 * j < NQ && q < NQ)
+                xq[q] = make_uint4(__byte_perm(ab0, cd0, 0x5410), __byte_perm(ab0, cd0, 0x7632),
+                                   __byte_perm(ab1, cd1, 0x5410), __byte_perm(ab1, cd1, 0x7632));
+        }
     }
 }
 
-template <int SYM, int GRP, int Q, bool PER>
-__global__ void __launch_bounds__(32 * GRP * Q) aeq_direct_kernel(const DevFrame *__restrict__ frames,
-                                                                   const AeqChain *__restrict__ chains,
-                                                                   AeqParams prm) {
-    using C = DirCfg<SYM, GRP, Q>;
-    constexpr int K = C::K, SA = C::SA, NS = C::NS;
-    __shared__ uint4 s_xq[C::XW];
+// e z of one output of a symbol: limbs c0 (16 bits), c1 (signed 16) and c2 with
+// e z = c2 2^32 + c1 2^16 + c0; c2 = 0 where e z fits 32 bits.  r2 <= 2^31 and
+// 18 A2 < 2^29 are exact in 32 bits unsigned, R - r2 in 32 bits signed.
+struct RdeLimbs {
+    uint32_t lo;
+    int32_t c2;
+};
+
+__device__ __forceinline__ RdeLimbs rde_limbs(int32_t z, int32_t zp, uint32_t A2, bool valid) {
+    const uint32_t r2 = (uint32_t)(z * z) + (uint32_t)(zp * zp);
+    const uint32_t R = 2 * A2 + (r2 < 6 * A2 ? 0 : 8 * A2) + (r2 < 14 * A2 ? 0 : 8 * A2);
+    const int32_t e = valid ? (int32_t)(R - r2) : 0;
+    const int64_t v = (int64_t)e * z;
+    return {(uint32_t)v, (int32_t)(v >> 32) + (int32_t)((uint32_t)v >> 31)};
+}
+
+// Limbs in shared memory, per output a row of NG groups of four symbols: ez holds
+// (c0 of symbols 0, 1; c0 of 2, 3; c1 of 0, 1; c1 of 2, 3), ez2 (c2 of 0, 1; of 2, 3).
+__device__ __forceinline__ void store_limbs(uint4 *ezrow, uint2 *ez2row, int si, RdeLimbs v) {
+    uint16_t *e16 = (uint16_t *)(ezrow + (si >> 2)) + (si & 3);
+    e16[0] = (uint16_t)v.lo;
+    e16[4] = (uint16_t)(v.lo >> 16);
+    ((uint16_t *)(ez2row + (si >> 2)))[si & 3] = (uint16_t)v.c2;
+}
+
+// Taps in shared memory, per output a row of eight 16-byte words: word
+// 4 (s1 / 2) + kg holds taps 4 kg + 3 .. 4 kg of inputs s1 and s1 + 1 in that order,
+// as they meet the bytes of xq.  Halfword of (s1, tap k) in the row:
+__device__ __forceinline__ int tap_slot(int s1, int k) {
+    return (s1 >> 1) * 32 + (k >> 2) * 8 + (s1 & 1) * 4 + 3 - (k & 3);
+}
+
+// Adds taps 4 kg .. 4 kg + 3 of the four inputs against x to two partial sums.
+__device__ __forceinline__ void conv4(const uint4 &wa, const uint4 &wb, const uint4 &x, int32_t &y0, int32_t &y1) {
+    y0 = dp2a<true, false>(wa.x, x.x, y0);
+    y1 = dp2a<true, true>(wa.y, x.x, y1);
+    y0 = dp2a<true, false>(wa.z, x.y, y0);
+    y1 = dp2a<true, true>(wa.w, x.y, y1);
+    y0 = dp2a<true, false>(wb.x, x.z, y0);
+    y1 = dp2a<true, true>(wb.y, x.z, y1);
+    y0 = dp2a<true, false>(wb.z, x.w, y0);
+    y1 = dp2a<true, true>(wb.w, x.w, y1);
+}
+
+// Four symbols of one input against the limbs c0, c1.
+__device__ __forceinline__ void grad4(const uint4 &e, uint32_t x, int32_t &l0, int32_t &l1) {
+    l0 = dp2a<false, false>(e.x, x, l0);
+    l1 = dp2a<true, false>(e.z, x, l1);
+    l0 = dp2a<false, true>(e.y, x, l0);
+    l1 = dp2a<true, true>(e.w, x, l1);
+}
+
+__device__ __forceinline__ int32_t out_of(int32_t y) { return min(max(y >> 7, -32768), 32767); }
+
+// ------------------------------------------------------------ few chains ----
+//
+// One CTA of five warps per (chain, polarisation).  Warps 0 .. SA / 16 - 1 form the
+// outputs (lane = 16 o + i: output o, symbol i of the warp's 16), so a convolution
+// needs no reduction; then all four consumer warps form the gradient and update the
+// taps of one input each (lane = 16 o + k: one tap a lane, whole block, no
+// reduction either).  Two barriers a block, of the four warps.  The fifth warp stages
+// and transposes the next batch into the other half of xq and meets the rest once a
+// batch.  What a block takes is latency: shared-memory loads, 32 dp2a, the error's
+// chain, SA dp2a, one 64-bit update.
+template <int NA, bool PER>
+__global__ void __launch_bounds__(160) aeq_split_kernel(const DevFrame *__restrict__ frames,
+                                                        const AeqChain *__restrict__ chains, AeqParams prm) {
+    using C = DirCfg<NA>;
+    constexpr int K = C::K, SA = C::SA, NG = C::NG, NC = SA / 16;
+    constexpr int WO = 12;                        // 16-byte words per tap row: the outputs 16 banks apart
+    __shared__ uint4 s_xq[2][C::XW];
     __shared__ uint32_t s_xn[C::XW];
-    // tap sets: GRP > 1 one per warp; Q > 1 two for the item, used in turn
-    __shared__ uint4 s_w[(GRP > 1 ? GRP : Q > 1 ? 2 : 1) * C::WS / 4];
-    // limbs of e z: [o][group of 4 symbols] (c0 01, c0 23, c1 01, c1 23); Q > 1: per warp
-    __shared__ uint4 s_ez[Q * 2 * C::NG];
-    __shared__ uint2 s_ez2[Q * 2 * C::NG];
-    __shared__ longlong2 s_part[GRP > 1 ? 2 * GRP * 64 : 1];   // partial gradients [parity][warp][pair][lane]
+    __shared__ uint4 s_w[2 * WO];
+    __shared__ uint4 s_ez[2 * NG];
+    __shared__ uint2 s_ez2[2 * NG];
+    __shared__ uint32_t s_big[4];
 
-    const int tid = threadIdx.x;
-    const int lane = tid & 31;
-    const int warp = tid >> 5;
-    const int grp = GRP > 1 ? warp : 0;
-    const int q4 = Q > 1 ? warp : 0;
-    const int o = lane >> 4, i = lane & 15;       // i: symbol of 16, then tap k
-    const uint32_t A2 = (uint32_t)prm.rde_a * (uint32_t)prm.rde_a;
-    const int mu = prm.mu_shift;
-    const int period = PER ? prm.period : 1;
-
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
     const AeqChain ch = chains[blockIdx.x >> 1];
     const int p = blockIdx.x & 1;
     const DevFrame &fr = frames[ch.frame];
     const uint32_t *xin = (const uint32_t *)fr.aeq_in;
-    int16_t *out = (int16_t *)fr.out;
+    const int64_t nblk = (ch.end - ch.begin + SA - 1) / SA;
+    const int64_t nbatch = (nblk + C::PB - 1) / C::PB;
 
-    uint32_t *wset = (uint32_t *)s_w + (GRP > 1 ? grp * C::WS : 0);
-    uint4 *ez = s_ez + q4 * 2 * C::NG;
-    uint2 *ez2 = s_ez2 + q4 * 2 * C::NG;
-    // tap k of (o, s1): halfword 3 - (k & 3) of the group of four taps k / 4
-    const int tapw = (o * C::WO + (i >> 2) * 8) * 2 + (3 - (i & 3));
-    int32_t T[NS];
-    int64_t acc[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        T[s] = ch.init[((2 * p + o) * 4 + q4 * NS + s) * K + i];
-        acc[s] = 0;
-        ((int16_t *)wset)[tapw + 4 * (q4 * NS + s)] = (int16_t)(T[s] >> 16);
+    if (warp == 4) {
+        stage<C>(s_xn, xin, ch.begin, ch.lo, ch.end, lane);
+        for (int64_t j = 0; j < nbatch; ++j) {
+            cp_async_wait_all();
+            __syncwarp();
+            transpose<C>(s_xn, s_xq[j & 1], lane);
+            __syncwarp();
+            if (j + 1 < nbatch) stage<C>(s_xn, xin, ch.begin + (j + 1) * C::B, ch.lo, ch.end, lane);
+            bar_sync<2, 160>();                   // batch j staged; batch j - 1 consumed
+        }
+        return;
     }
 
-    const int64_t nblk = (ch.end - ch.begin + SA - 1) / SA;
-    stage<C>(s_xn, xin, ch.begin, ch.lo, ch.end, tid);
+    const uint32_t A2 = (uint32_t)prm.rde_a * (uint32_t)prm.rde_a;
+    const int mu = prm.mu_shift;
+    const int o = lane >> 4, i = lane & 15;       // i: symbol of 16, then tap k
+    const int s1 = warp;
+    int16_t *wtap = (int16_t *)(s_w + o * WO) + tap_slot(s1, i);
+    int32_t T = ch.init[((2 * p + o) * 4 + s1) * K + i];
+    *wtap = (int16_t)(T >> 16);
+    if (lane == 0) s_big[warp] = 0;
+    int64_t acc = 0;
     int in_period = 0;
-    int par = 0;                                   // parity of the tap set (Q > 1) or the partial sums (GRP > 1)
+    for (int64_t j = 0; j < nbatch; ++j) {
+        bar_sync<2, 160>();
+        const int64_t tb = ch.begin + j * C::B;
+        const int nb = (int)min((int64_t)C::PB, nblk - j * C::PB);
+        // valid and kept symbols relative to the batch
+        const int rel_end = (int)min(ch.end - tb, (int64_t)C::B);
+        const int rel_keep = (int)min(max(ch.keep - tb, (int64_t)0), (int64_t)C::B);
+        int16_t *outb = (int16_t *)fr.out + tb * 4 + 2 * p;
+        for (int bb = 0; bb < nb; ++bb) {
+            const uint4 *xb = s_xq[j & 1] + K + bb * SA;
+
+            // ---- outputs: symbol 16 warp + i of output o
+            if (warp < NC) {
+                const uint4 *wr = s_w + o * WO;
+                int32_t y0 = 0, y1 = 0, y2 = 0, y3 = 0;
+#pragma unroll
+                for (int kg = 0; kg < 4; ++kg) {
+                    const uint4 x = xb[16 * warp + i - 4 * kg - 3];
+                    if (kg & 1)
+                        conv4(wr[kg], wr[4 + kg], x, y2, y3);
+                    else
+                        conv4(wr[kg], wr[4 + kg], x, y0, y1);
+                }
+                const int32_t z = out_of((y0 + y1) + (y2 + y3));
+                const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 16);
+                const int si = 16 * warp + i, rel = bb * SA + si;
+                const bool valid = rel < rel_end;
+                const RdeLimbs v = rde_limbs(z, zp, A2, valid);
+                store_limbs(s_ez + o * NG, s_ez2 + o * NG, si, v);
+                const bool any = __any_sync(0xffffffffu, v.c2 != 0);
+                if (lane == 0) s_big[warp] = any;
+                if (valid && rel >= rel_keep && o == 0)
+                    *(uint32_t *)(outb + rel * 4) = ((uint32_t)z & 0xFFFFu) | ((uint32_t)zp << 16);
+            }
+            if (mu >= 63) continue;                // the taps never move: no gradient
+
+            // ---- gradient of eq. (6) for (o, input s1, tap k = i)
+            const uint32_t *xs = (const uint32_t *)(xb - i) + s1;
+            uint32_t xg[NG];
+#pragma unroll
+            for (int n = 0; n < NG; ++n) xg[n] = xs[16 * n];
+            bar_sync<1, 128>();
+            int32_t l0 = 0, l1 = 0, m0 = 0, m1 = 0;
+#pragma unroll
+            for (int n = 0; n < NG; n += 2) {
+                grad4(s_ez[o * NG + n], xg[n], l0, l1);
+                grad4(s_ez[o * NG + n + 1], xg[n + 1], m0, m1);
+            }
+            int64_t g = (int64_t)(l1 + m1) * 65536 + (l0 + m0);
+            if (s_big[0] | s_big[1] | s_big[2]) {
+                int32_t l2 = 0;
+#pragma unroll
+                for (int n = 0; n < NG; ++n) {
+                    const uint2 e = s_ez2[o * NG + n];
+                    l2 = dp2a<true, false>(e.x, xg[n], l2);
+                    l2 = dp2a<true, true>(e.y, xg[n], l2);
+                }
+                g += (int64_t)l2 << 32;
+            }
+            bool apply = true;
+            if constexpr (PER) {
+                g = acc += g;
+                apply = ++in_period == prm.period || (j + 1 == nbatch && bb + 1 == nb);
+                if (apply) in_period = 0;
+            }
+            if (apply) {
+                T = add_tap(T, g >> mu);
+                *wtap = (int16_t)(T >> 16);
+                acc = 0;
+            }
+            bar_sync<1, 128>();                    // taps published, limbs free
+        }
+    }
+    if (ch.write_state) fr.state[((2 * p + o) * 4 + s1) * K + i] = T;
+}
+
+// ----------------------------------------------------------- many chains ----
+//
+// A warp per chain, both polarisations: lane = 8 S2 + i.  The lane forms symbols i,
+// i + 8, ... of output S2, then the gradient of taps i and i + 8 of S2 and all four
+// inputs over the block, and updates those eight taps.  Outputs and taps 8 apart
+// read the same staged words (4 apart by tap group), so a block of both
+// polarisations loads SA / 4 + 2 of them for each half of the work instead of SA / 4
+// and four per polarisation, group of 16 symbols and half: shared-memory loads
+// (two to four cycles each and SM) are what bounded a warp per (chain, polarisation).
+template <int NA, bool PER>
+__global__ void __launch_bounds__(32) aeq_pair_kernel(const DevFrame *__restrict__ frames,
+                                                      const AeqChain *__restrict__ chains, AeqParams prm) {
+    using C = DirCfg<NA>;
+    constexpr int K = C::K, SA = C::SA, NG = C::NG, M = SA / 8;
+    constexpr int WO = 10;                        // 16-byte words per tap row: rows 8 banks apart
+    constexpr int EO = NG + 2;                    // ... per limb row: rows 24 banks apart
+    __shared__ uint4 s_xq[C::XW];
+    __shared__ uint32_t s_xn[C::XW];
+    __shared__ uint4 s_w[4 * WO];
+    __shared__ uint4 s_ez[4 * EO];
+    __shared__ uint2 s_ez2[4 * EO];
+
+    const int lane = threadIdx.x;
+    const int S2 = lane >> 3, i = lane & 7;
+    const uint32_t A2 = (uint32_t)prm.rde_a * (uint32_t)prm.rde_a;
+    const int mu = prm.mu_shift;
+    const AeqChain ch = chains[blockIdx.x];
+    const DevFrame &fr = frames[ch.frame];
+    const uint32_t *xin = (const uint32_t *)fr.aeq_in;
+
+    int16_t *wrow = (int16_t *)(s_w + S2 * WO);
+    int32_t T[2][4];
+    int64_t acc[PER ? 2 : 1][4];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            T[c][s] = ch.init[(S2 * 4 + s) * K + i + 8 * c];
+            wrow[tap_slot(s, i + 8 * c)] = (int16_t)(T[c][s] >> 16);
+            if (PER) acc[c][s] = 0;
+        }
+
+    const int64_t nblk = (ch.end - ch.begin + SA - 1) / SA;
+    stage<C>(s_xn, xin, ch.begin, ch.lo, ch.end, lane);
+    int in_period = 0;
     for (int64_t b0 = 0; b0 < nblk; b0 += C::PB) {
         const int64_t tb = ch.begin + b0 * SA;
         cp_async_wait_all();
-        item_sync<C::W>();                         // words staged; the last batch's reads of xq done
-        transpose<C>(s_xn, s_xq, tid);
-        item_sync<C::W>();
-        if (b0 + C::PB < nblk) stage<C>(s_xn, xin, tb + C::B, ch.lo, ch.end, tid);
+        __syncwarp();
+        transpose<C>(s_xn, s_xq, lane);
+        __syncwarp();
+        if (b0 + C::PB < nblk) stage<C>(s_xn, xin, tb + C::B, ch.lo, ch.end, lane);
         const int nb = (int)min((int64_t)C::PB, nblk - b0);
         const bool last_batch = b0 + C::PB >= nblk;
         // valid and kept symbols relative to the batch
         const int rel_end = (int)min(ch.end - tb, (int64_t)C::B);
         const int rel_keep = (int)min(max(ch.keep - tb, (int64_t)0), (int64_t)C::B);
-        int16_t *outb = out + tb * 4 + 2 * p;
+        int16_t *outb = (int16_t *)fr.out + tb * 4 + (S2 & 2);
         for (int bb = 0; bb < nb; ++bb) {
             const uint4 *xb = s_xq + K + bb * SA;
 
-            // ---- convolution: y of (o, symbol 16 (grp SYM + m) + i)
-            const uint4 *wr = (const uint4 *)(wset + (Q > 1 ? par * C::WS : 0) + o * C::WO);
-            int32_t y[SYM][2];
+            // ---- convolution: symbol i + 8 m, tap group kg read word i - 15 + 4 (2 m + 3 - kg)
+            int32_t y0[M], y1[M];
+            {
+                const uint4 *wr = s_w + S2 * WO;
+                uint4 wa[4], wb[4];
 #pragma unroll
-            for (int m = 0; m < SYM; ++m) y[m][0] = y[m][1] = 0;
+                for (int kg = 0; kg < 4; ++kg) {
+                    wa[kg] = wr[kg];
+                    wb[kg] = wr[4 + kg];
+                }
 #pragma unroll
-            for (int kg = 0; kg < 4; ++kg) {
-                const uint4 wa = wr[2 * kg], wb = wr[2 * kg + 1];
+                for (int m = 0; m < M; ++m) y0[m] = y1[m] = 0;
 #pragma unroll
-                for (int m = 0; m < SYM; ++m) {
-                    const uint4 x = xb[16 * (grp * SYM + m) + i - 4 * kg - 3];
-                    y[m][0] = dp2a<true, false>(wa.x, x.x, y[m][0]);
-                    y[m][1] = dp2a<true, true>(wa.y, x.x, y[m][1]);
-                    y[m][0] = dp2a<true, false>(wa.z, x.y, y[m][0]);
-                    y[m][1] = dp2a<true, true>(wa.w, x.y, y[m][1]);
-                    y[m][0] = dp2a<true, false>(wb.x, x.z, y[m][0]);
-                    y[m][1] = dp2a<true, true>(wb.y, x.z, y[m][1]);
-                    y[m][0] = dp2a<true, false>(wb.z, x.w, y[m][0]);
-                    y[m][1] = dp2a<true, true>(wb.w, x.w, y[m][1]);
+                for (int j = 0; j < 2 * M + 2; ++j) {
+                    const uint4 x = xb[i - 15 + 4 * j];
+#pragma unroll
+                    for (int m = 0; m < M; ++m) {
+                        const int kg = 2 * m + 3 - j;
+                        if (kg >= 0 && kg < 4) conv4(wa[kg & 3], wb[kg & 3], x, y0[m], y1[m]);
+                    }
                 }
             }
 
             // ---- outputs, RDE error, limbs of e z
             bool big = false;
 #pragma unroll
-            for (int m = 0; m < SYM; ++m) {
-                const int si = 16 * (grp * SYM + m) + i;
-                const int32_t z = min(max((y[m][0] + y[m][1]) >> 7, -32768), 32767);
-                const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 16);
-                // r2 <= 2^31 and 18 A2 < 2^29: exact in 32 bits unsigned
-                const uint32_t r2 = (uint32_t)(z * z) + (uint32_t)(zp * zp);
-                const uint32_t Rr = r2 < 6 * A2 ? 2 * A2 : (r2 < 14 * A2 ? 10 * A2 : 18 * A2);
-                const int rel = bb * SA + si;
+            for (int m = 0; m < M; ++m) {
+                const int si = i + 8 * m, rel = bb * SA + si;
+                const int32_t z = out_of(y0[m] + y1[m]);
+                const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 8);
                 const bool valid = rel < rel_end;
-                if (valid && rel >= rel_keep && o == 0 && q4 == 0)
+                const RdeLimbs v = rde_limbs(z, zp, A2, valid);
+                store_limbs(s_ez + S2 * EO, s_ez2 + S2 * EO, si, v);
+                big |= v.c2 != 0;
+                if (valid && rel >= rel_keep && (S2 & 1) == 0)
                     *(uint32_t *)(outb + rel * 4) = ((uint32_t)z & 0xFFFFu) | ((uint32_t)zp << 16);
-                const int64_t v = valid ? (int64_t)(int32_t)(Rr - r2) * z : 0;
-                // e z = c2 2^32 + c1 2^16 + c0 with c1 signed: c2 is 0 where e z fits 32 bits
-                const uint32_t vl = (uint32_t)v;
-                const int32_t c2 = (int32_t)(v >> 32) + (int32_t)(vl >> 31);
-                big |= c2 != 0;
-                uint16_t *e16 = (uint16_t *)(ez + o * C::NG + (si >> 2)) + (si & 3);
-                e16[0] = (uint16_t)vl;
-                e16[4] = (uint16_t)(vl >> 16);
-                ((uint16_t *)(ez2 + o * C::NG + (si >> 2)))[si & 3] = (uint16_t)c2;
             }
-            // (also orders the limbs before the gradient's reads, within the warp)
             const bool any = __any_sync(0xffffffffu, big);
             __syncwarp();
+            if (mu >= 63) continue;                // the taps never move: no gradient
 
-            // ---- gradient of eq. (6) for (o, s1, tap k = i) over the warp's symbols
-            if (mu < 63) {
-                int32_t l0[NS], l1[NS];
-                int64_t g[NS];
+            // ---- gradient of eq. (6): tap i + 8 c, symbol group n read word
+            // -i - 8 + 4 (n - 2 c + 2)
+            int32_t l0[2][4], l1[2][4];
 #pragma unroll
-                for (int s = 0; s < NS; ++s) l0[s] = l1[s] = 0;
+            for (int c = 0; c < 2; ++c)
 #pragma unroll
-                for (int n = 0; n < 4 * SYM; ++n) {
-                    const int ig = 4 * SYM * grp + n;
-                    const uint4 e = ez[o * C::NG + ig];
-                    const uint4 x = xb[4 * ig - i];
+                for (int s = 0; s < 4; ++s) l0[c][s] = l1[c][s] = 0;
+            const uint4 *er = s_ez + S2 * EO;
+            uint4 e0 = er[0], e1 = er[0], e2;      // limbs of groups j, j - 1, j - 2
 #pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        const uint32_t xs = Q == 1 ? word_of(x, s) : ((const uint32_t *)(xb + 4 * ig - i))[q4 * NS + s];
-                        l0[s] = dp2a<false, false>(e.x, xs, l0[s]);
-                        l1[s] = dp2a<true, false>(e.z, xs, l1[s]);
-                        l0[s] = dp2a<false, true>(e.y, xs, l0[s]);
-                        l1[s] = dp2a<true, true>(e.w, xs, l1[s]);
-                    }
-                }
+            for (int j = 0; j < NG + 2; ++j) {
+                e2 = e1;
+                e1 = e0;
+                if (j < NG) e0 = er[j];
+                const uint4 x = xb[4 * j - 8 - i];
 #pragma unroll
-                for (int s = 0; s < NS; ++s) g[s] = (int64_t)l1[s] * 65536 + l0[s];
-                if (any) {
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        int32_t l2 = 0;
-                        for (int n = 0; n < 4 * SYM; ++n) {
-                            const int ig = 4 * SYM * grp + n;
-                            const uint2 e = ez2[o * C::NG + ig];
-                            const uint32_t xs = ((const uint32_t *)(xb + 4 * ig - i))[q4 * NS + s];
-                            l2 = dp2a<true, false>(e.x, xs, l2);
-                            l2 = dp2a<true, true>(e.y, xs, l2);
-                        }
-                        g[s] += (int64_t)l2 << 32;
-                    }
-                }
-                bool apply = true;
-                if constexpr (PER) {
-                    apply = ++in_period == period || (last_batch && bb + 1 == nb);
-                    if (apply) in_period = 0;
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) g[s] = acc[s] += g[s];
-                }
-                if (apply) {
-                    if constexpr (GRP > 1) {
-                        // the other warps' partial sums over the period; two buffers in
-                        // turn, so one barrier an update
-                        longlong2 *part = s_part + par * GRP * 64;
-                        part[grp * 64 + lane] = make_longlong2(g[0], g[1]);
-                        part[grp * 64 + 32 + lane] = make_longlong2(g[2], g[3]);
-                        __syncthreads();
-#pragma unroll
-                        for (int w = 1; w < GRP; ++w) {
-                            const int og = grp + w < GRP ? grp + w : grp + w - GRP;
-                            const longlong2 u = part[og * 64 + lane], v = part[og * 64 + 32 + lane];
-                            g[0] += u.x;
-                            g[1] += u.y;
-                            g[2] += v.x;
-                            g[3] += v.y;
-                        }
-                    }
-                    if constexpr (GRP > 1 || Q > 1) par ^= 1;
-                    int16_t *wn = (int16_t *)(wset + (Q > 1 ? par * C::WS : 0));
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        T[s] = add_tap(T[s], g[s] >> mu);
-                        wn[tapw + 4 * (q4 * NS + s)] = (int16_t)(T[s] >> 16);
-                        acc[s] = 0;
-                    }
-                    item_sync<Q>();                // the item's new taps, before the next block reads them
-                } else {
-                    __syncwarp();                  // the limbs are rewritten by the next block
+                for (int s = 0; s < 4; ++s) {
+                    if (j >= 2) grad4(e2, word_of(x, s), l0[0][s], l1[0][s]);
+                    if (j < NG) grad4(e0, word_of(x, s), l0[1][s], l1[1][s]);
                 }
             }
+            int64_t g[2][4];
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int s = 0; s < 4; ++s) g[c][s] = (int64_t)l1[c][s] * 65536 + l0[c][s];
+            if (any) {
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    int32_t l2[4] = {0, 0, 0, 0};
+                    for (int n = 0; n < NG; ++n) {
+                        const uint2 e = s_ez2[S2 * EO + n];
+                        const uint4 x = xb[4 * n - 8 * c - i];
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) {
+                            l2[s] = dp2a<true, false>(e.x, word_of(x, s), l2[s]);
+                            l2[s] = dp2a<true, true>(e.y, word_of(x, s), l2[s]);
+                        }
+                    }
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) g[c][s] += (int64_t)l2[s] << 32;
+                }
+            }
+            bool apply = true;
+            if constexpr (PER) {
+                apply = ++in_period == prm.period || (last_batch && bb + 1 == nb);
+                if (apply) in_period = 0;
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) g[c][s] = acc[c][s] += g[c][s];
+            }
+            if (apply) {
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) {
+                        T[c][s] = add_tap(T[c][s], g[c][s] >> mu);
+                        wrow[tap_slot(s, i + 8 * c)] = (int16_t)(T[c][s] >> 16);
+                        if (PER) acc[c][s] = 0;
+                    }
+            }
+            __syncwarp();                          // taps published, limbs free
         }
     }
-    if (ch.write_state && grp == 0) {
+    if (ch.write_state) {
 #pragma unroll
-        for (int s = 0; s < NS; ++s) fr.state[((2 * p + o) * 4 + q4 * NS + s) * K + i] = T[s];
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) fr.state[(S2 * 4 + s) * K + i + 8 * c] = T[c][s];
     }
 }
 
-template <int SYM, int GRP, int Q>
-cudaError_t launch_layout(const DevFrame *frames, const AeqChain *chains, int n_chains, AeqParams prm,
-                          cudaStream_t stream) {
-    const unsigned grid = 2u * (unsigned)n_chains;
-    if (prm.period > 1)
-        aeq_direct_kernel<SYM, GRP, Q, true><<<grid, 32 * GRP * Q, 0, stream>>>(frames, chains, prm);
+template <int NA>
+void launch_na(bool split, const DevFrame *frames, const AeqChain *chains, int n_chains, AeqParams prm,
+               cudaStream_t stream) {
+    const unsigned n = (unsigned)n_chains;
+    if (split && prm.period > 1)
+        aeq_split_kernel<NA, true><<<2 * n, 160, 0, stream>>>(frames, chains, prm);
+    else if (split)
+        aeq_split_kernel<NA, false><<<2 * n, 160, 0, stream>>>(frames, chains, prm);
+    else if (prm.period > 1)
+        aeq_pair_kernel<NA, true><<<n, 32, 0, stream>>>(frames, chains, prm);
     else
-        aeq_direct_kernel<SYM, GRP, Q, false><<<grid, 32 * GRP * Q, 0, stream>>>(frames, chains, prm);
-    return cudaGetLastError();
+        aeq_pair_kernel<NA, false><<<n, 32, 0, stream>>>(frames, chains, prm);
 }
 
 }  // namespace
 
+// The split layout takes fewer cycles a block while the GPU is not full; the pair
+// layout fewer cycles of an SM a block.  total / longest is how many chains of the
+// longest one's length the launch amounts to.
 cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
                               int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
                               cudaStream_t stream) {
     if (n_chains <= 0) return cudaSuccess;
-    const bool spread = 2.0 * total_symbols < 8.0 * n_sm * (double)longest_symbols;
+    const double items = 2.0 * (double)total_symbols / (double)std::max<int64_t>(longest_symbols, 1);
+    const bool split = items < (na == 64 ? 5.0 : 7.0) * n_sm;
     if (na == 64)
-        return spread ? launch_layout<1, 3, 1>(frames, chains, n_chains, prm, stream)
-                      : launch_layout<3, 1, 1>(frames, chains, n_chains, prm, stream);
-    return spread ? launch_layout<1, 1, 4>(frames, chains, n_chains, prm, stream)
-                  : launch_layout<1, 1, 1>(frames, chains, n_chains, prm, stream);
+        launch_na<64>(split, frames, chains, n_chains, prm, stream);
+    else
+        launch_na<32>(split, frames, chains, n_chains, prm, stream);
+    return cudaGetLastError();
 }
 
 }  // namespace fnt
