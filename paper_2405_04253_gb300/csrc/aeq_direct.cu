@@ -30,8 +30,8 @@
 // Two layouts; aeq_direct_launch picks one (rule and figures there).
 //   aeq_pair_kernel   a warp per chain, both polarisations: many chains, bound by
 //                     dp2a issue and shared-memory loads
-//   aeq_split_kernel  five warps per (chain, polarisation): few chains, bound by the
-//                     latency of one block
+//   aeq_split_kernel  six or eight warps per (chain, polarisation), by role: few
+//                     chains, bound by the latency of one block
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -95,6 +95,21 @@ __device__ __forceinline__ int32_t add_tap(int32_t T, int64_t d) {
     return min(max(w, -(1 << 29)), (1 << 29) - 1);
 }
 
+// add_tap(T, g >> mu) for g = l1 2^16 + l0 with |l1| < 2^26 and T inside the 30-bit
+// range, in 32 bits: g = h 2^16 + r, 0 <= r < 2^16.  Below mu = 16 the step is h 2^(16-mu)
+// plus r's top bits, h first cut to where the sum is past the range anyway.
+__device__ __forceinline__ int32_t add_tap32(int32_t T, int32_t l1, int32_t l0, int mu) {
+    const int32_t h = l1 + (l0 >> 16);
+    int32_t d;
+    if (mu >= 16)
+        d = h >> min(mu - 16, 31);
+    else
+        d = (min(max(h, -(3 << (13 + mu))), 1 << (14 + mu)) << (16 - mu)) + ((l0 & 0xFFFF) >> mu);
+    return min(max(T + d, -(1 << 29)), (1 << 29) - 1);
+}
+
+__device__ __forceinline__ bool tap_in_range(int32_t T) { return T >= -(1 << 29) && T < (1 << 29); }
+
 // A warp's copies of symbols tb - K + q, q < XW (zero outside [lo, end)), to xn.
 template <class C>
 __device__ __forceinline__ void stage(uint32_t *xn, const uint32_t *xin, int64_t tb, int64_t lo, int64_t end,
@@ -154,10 +169,13 @@ __device__ __forceinline__ RdeLimbs rde_limbs(int32_t z, int32_t zp, uint32_t A2
 
 // Limbs in shared memory, per output a row of NG groups of four symbols: ez holds
 // (c0 of symbols 0, 1; c0 of 2, 3; c1 of 0, 1; c1 of 2, 3), ez2 (c2 of 0, 1; of 2, 3).
-__device__ __forceinline__ void store_limbs(uint4 *ezrow, uint2 *ez2row, int si, RdeLimbs v) {
+__device__ __forceinline__ void store_limbs(uint4 *ezrow, int si, RdeLimbs v) {
     uint16_t *e16 = (uint16_t *)(ezrow + (si >> 2)) + (si & 3);
     e16[0] = (uint16_t)v.lo;
     e16[4] = (uint16_t)(v.lo >> 16);
+}
+
+__device__ __forceinline__ void store_limb2(uint2 *ez2row, int si, RdeLimbs v) {
     ((uint16_t *)(ez2row + (si >> 2)))[si & 3] = (uint16_t)v.c2;
 }
 
@@ -192,26 +210,45 @@ __device__ __forceinline__ int32_t out_of(int32_t y) { return min(max(y >> 7, -3
 
 // ------------------------------------------------------------ few chains ----
 //
-// One CTA of five warps per (chain, polarisation).  Warps 0 .. SA / 16 - 1 form the
-// outputs (lane = 16 o + i: output o, symbol i of the warp's 16), so a convolution
-// needs no reduction; then all four consumer warps form the gradient and update the
-// taps of one input each (lane = 16 o + k: one tap a lane, whole block, no
-// reduction either).  Two barriers a block, of the four warps.  The fifth warp stages
-// and transposes the next batch into the other half of xq and meets the rest once a
-// batch.  What a block takes is latency: shared-memory loads, 32 dp2a, the error's
-// chain, SA dp2a, one 64-bit update.
+// One CTA per (chain, polarisation), its warps by role, so that only what the next
+// step waits for lies between two of them:
+//   NC = SA / 16 output warps: lane = 16 o + i, output o, symbol i of the warp's 16
+//     (no reduction), the error and the limbs of e z; between blocks they store the
+//     outputs and load the next block's symbols
+//   4 gradient warps, one per input s1: lane = 16 o + k, the gradient of one tap over
+//     the block and its update; between blocks they load the next block's symbols
+//   1 staging warp: the next batch into the other half of xq, once a batch
+// Limbs go from output to gradient warps at barrier 1, taps back at barrier 3 (the
+// writers arrive, the readers wait); barrier 2 joins all warps once a batch.
+// What a block takes is the latency of that round trip: about 200 instructions a warp
+// at 3 to 4 cycles each when one warp held a whole block.
+template <int NA>
+struct SplitCfg {
+    static constexpr int NC = (NA - kAeqK) / 16;          // output warps
+    static constexpr int NGW = 4;                         // gradient warps
+    static constexpr int NCG = 32 * (NC + NGW);
+    static constexpr int NT = NCG + 32;
+};
+
+template <int ID, int N>
+__device__ __forceinline__ void bar_arrive() {
+    asm volatile("bar.arrive %0, %1;\n" ::"n"(ID), "n"(N) : "memory");
+}
+
 template <int NA, bool PER>
-__global__ void __launch_bounds__(160) aeq_split_kernel(const DevFrame *__restrict__ frames,
-                                                        const AeqChain *__restrict__ chains, AeqParams prm) {
+__global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFrame *__restrict__ frames,
+                                                                     const AeqChain *__restrict__ chains,
+                                                                     AeqParams prm) {
     using C = DirCfg<NA>;
-    constexpr int K = C::K, SA = C::SA, NG = C::NG, NC = SA / 16;
+    using R = SplitCfg<NA>;
+    constexpr int K = C::K, SA = C::SA, NG = C::NG, NC = R::NC, NCG = R::NCG;
     constexpr int WO = 12;                        // 16-byte words per tap row: the outputs 16 banks apart
     __shared__ uint4 s_xq[2][C::XW];
     __shared__ uint32_t s_xn[C::XW];
     __shared__ uint4 s_w[2 * WO];
     __shared__ uint4 s_ez[2 * NG];
     __shared__ uint2 s_ez2[2 * NG];
-    __shared__ uint32_t s_big[4];
+    __shared__ uint4 s_big;                       // word w: output warp w stored third limbs
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -221,8 +258,12 @@ __global__ void __launch_bounds__(160) aeq_split_kernel(const DevFrame *__restri
     const uint32_t *xin = (const uint32_t *)fr.aeq_in;
     const int64_t nblk = (ch.end - ch.begin + SA - 1) / SA;
     const int64_t nbatch = (nblk + C::PB - 1) / C::PB;
+    const int mu = prm.mu_shift;
+    const int o = lane >> 4, i = lane & 15;
 
-    if (warp == 4) {
+    if (warp == NC + R::NGW) {
+        // ---- staging
+        if (lane == 0) s_big = make_uint4(0, 0, 0, 0);
         stage<C>(s_xn, xin, ch.begin, ch.lo, ch.end, lane);
         for (int64_t j = 0; j < nbatch; ++j) {
             cp_async_wait_all();
@@ -230,95 +271,115 @@ __global__ void __launch_bounds__(160) aeq_split_kernel(const DevFrame *__restri
             transpose<C>(s_xn, s_xq[j & 1], lane);
             __syncwarp();
             if (j + 1 < nbatch) stage<C>(s_xn, xin, ch.begin + (j + 1) * C::B, ch.lo, ch.end, lane);
-            bar_sync<2, 160>();                   // batch j staged; batch j - 1 consumed
+            bar_sync<2, R::NT>();                 // batch j staged; batch j - 1 consumed
         }
-        return;
-    }
-
-    const uint32_t A2 = (uint32_t)prm.rde_a * (uint32_t)prm.rde_a;
-    const int mu = prm.mu_shift;
-    const int o = lane >> 4, i = lane & 15;       // i: symbol of 16, then tap k
-    const int s1 = warp;
-    int16_t *wtap = (int16_t *)(s_w + o * WO) + tap_slot(s1, i);
-    int32_t T = ch.init[((2 * p + o) * 4 + s1) * K + i];
-    *wtap = (int16_t)(T >> 16);
-    if (lane == 0) s_big[warp] = 0;
-    int64_t acc = 0;
-    int in_period = 0;
-    for (int64_t j = 0; j < nbatch; ++j) {
-        bar_sync<2, 160>();
-        const int64_t tb = ch.begin + j * C::B;
-        const int nb = (int)min((int64_t)C::PB, nblk - j * C::PB);
-        // valid and kept symbols relative to the batch
-        const int rel_end = (int)min(ch.end - tb, (int64_t)C::B);
-        const int rel_keep = (int)min(max(ch.keep - tb, (int64_t)0), (int64_t)C::B);
-        int16_t *outb = (int16_t *)fr.out + tb * 4 + 2 * p;
-        for (int bb = 0; bb < nb; ++bb) {
-            const uint4 *xb = s_xq[j & 1] + K + bb * SA;
-
-            // ---- outputs: symbol 16 warp + i of output o
-            if (warp < NC) {
-                const uint4 *wr = s_w + o * WO;
-                int32_t y0 = 0, y1 = 0, y2 = 0, y3 = 0;
+    } else if (warp < NC) {
+        // ---- outputs: symbol si of output o
+        const uint32_t A2 = (uint32_t)prm.rde_a * (uint32_t)prm.rde_a;
+        const int si = 16 * warp + i;
+        const uint4 *wr = s_w + o * WO;
+        for (int64_t j = 0; j < nbatch; ++j) {
+            bar_sync<2, R::NT>();                 // (j = 0: also the initial taps)
+            const int64_t tb = ch.begin + j * C::B;
+            const int nb = (int)min((int64_t)C::PB, nblk - j * C::PB);
+            // valid and kept symbols relative to the batch, less the lane's
+            const int left = (int)min(ch.end - tb, (int64_t)C::B) - si;
+            const int skip = (int)min(max(ch.keep - tb, (int64_t)0), (int64_t)C::B) - si;
+            int16_t *dst = (int16_t *)fr.out + (tb + si) * 4 + 2 * p;
+            const uint4 *xb = s_xq[j & 1] + K + si - 3;
+            uint4 x[4];                           // a block ahead
+#pragma unroll
+            for (int kg = 0; kg < 4; ++kg) x[kg] = xb[-4 * kg];
+            for (int bb = 0; bb < nb; ++bb) {
+                const bool valid = bb * SA < left;
+                int32_t y[4][2];
 #pragma unroll
                 for (int kg = 0; kg < 4; ++kg) {
-                    const uint4 x = xb[16 * warp + i - 4 * kg - 3];
-                    if (kg & 1)
-                        conv4(wr[kg], wr[4 + kg], x, y2, y3);
-                    else
-                        conv4(wr[kg], wr[4 + kg], x, y0, y1);
+                    y[kg][0] = y[kg][1] = 0;
+                    conv4(wr[kg], wr[4 + kg], x[kg], y[kg][0], y[kg][1]);
                 }
-                const int32_t z = out_of((y0 + y1) + (y2 + y3));
+                const int32_t z =
+                    out_of(((y[0][0] + y[0][1]) + (y[1][0] + y[1][1])) + ((y[2][0] + y[2][1]) + (y[3][0] + y[3][1])));
                 const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 16);
-                const int si = 16 * warp + i, rel = bb * SA + si;
-                const bool valid = rel < rel_end;
-                const RdeLimbs v = rde_limbs(z, zp, A2, valid);
-                store_limbs(s_ez + o * NG, s_ez2 + o * NG, si, v);
-                const bool any = __any_sync(0xffffffffu, v.c2 != 0);
-                if (lane == 0) s_big[warp] = any;
-                if (valid && rel >= rel_keep && o == 0)
-                    *(uint32_t *)(outb + rel * 4) = ((uint32_t)z & 0xFFFFu) | ((uint32_t)zp << 16);
-            }
-            if (mu >= 63) continue;                // the taps never move: no gradient
-
-            // ---- gradient of eq. (6) for (o, input s1, tap k = i)
-            const uint32_t *xs = (const uint32_t *)(xb - i) + s1;
-            uint32_t xg[NG];
-#pragma unroll
-            for (int n = 0; n < NG; ++n) xg[n] = xs[16 * n];
-            bar_sync<1, 128>();
-            int32_t l0 = 0, l1 = 0, m0 = 0, m1 = 0;
-#pragma unroll
-            for (int n = 0; n < NG; n += 2) {
-                grad4(s_ez[o * NG + n], xg[n], l0, l1);
-                grad4(s_ez[o * NG + n + 1], xg[n + 1], m0, m1);
-            }
-            int64_t g = (int64_t)(l1 + m1) * 65536 + (l0 + m0);
-            if (s_big[0] | s_big[1] | s_big[2]) {
-                int32_t l2 = 0;
-#pragma unroll
-                for (int n = 0; n < NG; ++n) {
-                    const uint2 e = s_ez2[o * NG + n];
-                    l2 = dp2a<true, false>(e.x, xg[n], l2);
-                    l2 = dp2a<true, true>(e.y, xg[n], l2);
+                if (mu < 63) {
+                    const RdeLimbs v = rde_limbs(z, zp, A2, valid);
+                    store_limbs(s_ez + o * NG, si, v);
+                    const bool any = __any_sync(0xffffffffu, v.c2 != 0);
+                    if (any) store_limb2(s_ez2 + o * NG, si, v);
+                    if (lane == 0) ((uint32_t *)&s_big)[warp] = any;
+                    bar_arrive<1, NCG>();          // limbs stored
                 }
-                g += (int64_t)l2 << 32;
+                xb += SA;
+                if (bb + 1 < nb) {
+#pragma unroll
+                    for (int kg = 0; kg < 4; ++kg) x[kg] = xb[-4 * kg];
+                }
+                if (o == 0 && valid && bb * SA >= skip)
+                    *(uint32_t *)(dst + bb * SA * 4) = ((uint32_t)z & 0xFFFFu) | ((uint32_t)zp << 16);
+                if (mu < 63) bar_sync<3, NCG>();   // taps published, limbs free
             }
-            bool apply = true;
-            if constexpr (PER) {
-                g = acc += g;
-                apply = ++in_period == prm.period || (j + 1 == nbatch && bb + 1 == nb);
-                if (apply) in_period = 0;
-            }
-            if (apply) {
-                T = add_tap(T, g >> mu);
-                *wtap = (int16_t)(T >> 16);
-                acc = 0;
-            }
-            bar_sync<1, 128>();                    // taps published, limbs free
         }
+    } else {
+        // ---- gradient of eq. (6) and update: tap k = i of (o, input s1)
+        const int s1 = warp - NC;
+        int16_t *wtap = (int16_t *)(s_w + o * WO) + tap_slot(s1, i);
+        int32_t T = ch.init[((2 * p + o) * 4 + s1) * K + i];
+        *wtap = (int16_t)(T >> 16);
+        bool wide = !tap_in_range(T);              // a caller's state, until the first update
+        int64_t acc = 0;
+        int in_period = 0;
+        const uint4 *er = s_ez + o * NG;
+        for (int64_t j = 0; j < nbatch; ++j) {
+            bar_sync<2, R::NT>();
+            if (mu >= 63) continue;                // the taps never move
+            const int nb = (int)min((int64_t)C::PB, nblk - j * C::PB);
+            const uint32_t *xs = (const uint32_t *)(s_xq[j & 1] + K - i) + s1;
+            for (int bb = 0; bb < nb; ++bb, xs += 4 * SA) {
+                uint32_t x[NG];
+#pragma unroll
+                for (int n = 0; n < NG; ++n) x[n] = xs[16 * n];
+                bar_sync<1, NCG>();                // limbs stored
+                int32_t l0[4] = {0, 0, 0, 0}, l1[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int n = 0; n < NG; ++n) grad4(er[n], x[n], l0[n & 3], l1[n & 3]);
+                const uint4 big = s_big;
+                const bool any = NC == 1 ? big.x != 0 : (big.x | big.y | big.z) != 0;
+                const int32_t g0 = (l0[0] + l0[1]) + (l0[2] + l0[3]), g1 = (l1[0] + l1[1]) + (l1[2] + l1[3]);
+                if (!PER && !any && !wide) {
+                    T = add_tap32(T, g1, g0, mu);
+                    *wtap = (int16_t)(T >> 16);
+                } else {
+                    int64_t g = (int64_t)g1 * 65536 + g0;
+                    if (any) {
+                        int32_t l2 = 0;
+#pragma unroll
+                        for (int n = 0; n < NG; ++n) {
+                            if (word_of(big, n / 4) == 0) continue;   // that warp's are all 0, not stored
+                            const uint2 e = s_ez2[o * NG + n];
+                            l2 = dp2a<true, false>(e.x, x[n], l2);
+                            l2 = dp2a<true, true>(e.y, x[n], l2);
+                        }
+                        g += (int64_t)l2 << 32;
+                    }
+                    bool apply = true;
+                    if constexpr (PER) {
+                        g += acc;
+                        apply = ++in_period == prm.period || (j + 1 == nbatch && bb + 1 == nb);
+                        if (apply) in_period = 0;
+                        acc = apply ? 0 : g;
+                    }
+                    if (apply) {
+                        T = add_tap(T, g >> mu);
+                        *wtap = (int16_t)(T >> 16);
+                        wide = false;
+                    }
+                }
+                __syncwarp();
+                bar_arrive<3, NCG>();              // taps published, limbs read
+            }
+        }
+        if (ch.write_state) fr.state[((2 * p + o) * 4 + s1) * K + i] = T;
     }
-    if (ch.write_state) fr.state[((2 * p + o) * 4 + s1) * K + i] = T;
 }
 
 // ----------------------------------------------------------- many chains ----
@@ -354,14 +415,18 @@ __global__ void __launch_bounds__(32) aeq_pair_kernel(const DevFrame *__restrict
     int16_t *wrow = (int16_t *)(s_w + S2 * WO);
     int32_t T[2][4];
     int64_t acc[PER ? 2 : 1][4];
+    bool wide = false;   // a caller's state may hold taps beyond the 30-bit range until the first update
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             T[c][s] = ch.init[(S2 * 4 + s) * K + i + 8 * c];
+            wide |= !tap_in_range(T[c][s]);
             wrow[tap_slot(s, i + 8 * c)] = (int16_t)(T[c][s] >> 16);
             if (PER) acc[c][s] = 0;
         }
+
+    wide = __any_sync(0xffffffffu, wide);
 
     const int64_t nblk = (ch.end - ch.begin + SA - 1) / SA;
     stage<C>(s_xn, xin, ch.begin, ch.lo, ch.end, lane);
@@ -407,19 +472,24 @@ __global__ void __launch_bounds__(32) aeq_pair_kernel(const DevFrame *__restrict
 
             // ---- outputs, RDE error, limbs of e z
             bool big = false;
+            RdeLimbs v[M];
 #pragma unroll
             for (int m = 0; m < M; ++m) {
                 const int si = i + 8 * m, rel = bb * SA + si;
                 const int32_t z = out_of(y0[m] + y1[m]);
                 const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 8);
                 const bool valid = rel < rel_end;
-                const RdeLimbs v = rde_limbs(z, zp, A2, valid);
-                store_limbs(s_ez + S2 * EO, s_ez2 + S2 * EO, si, v);
-                big |= v.c2 != 0;
+                v[m] = rde_limbs(z, zp, A2, valid);
+                store_limbs(s_ez + S2 * EO, si, v[m]);
+                big |= v[m].c2 != 0;
                 if (valid && rel >= rel_keep && (S2 & 1) == 0)
                     *(uint32_t *)(outb + rel * 4) = ((uint32_t)z & 0xFFFFu) | ((uint32_t)zp << 16);
             }
             const bool any = __any_sync(0xffffffffu, big);
+            if (any) {
+#pragma unroll
+                for (int m = 0; m < M; ++m) store_limb2(s_ez2 + S2 * EO, i + 8 * m, v[m]);
+            }
             __syncwarp();
             if (mu >= 63) continue;                // the taps never move: no gradient
 
@@ -444,46 +514,47 @@ __global__ void __launch_bounds__(32) aeq_pair_kernel(const DevFrame *__restrict
                     if (j < NG) grad4(e0, word_of(x, s), l0[1][s], l1[1][s]);
                 }
             }
-            int64_t g[2][4];
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int s = 0; s < 4; ++s) g[c][s] = (int64_t)l1[c][s] * 65536 + l0[c][s];
-            if (any) {
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    int32_t l2[4] = {0, 0, 0, 0};
-                    for (int n = 0; n < NG; ++n) {
-                        const uint2 e = s_ez2[S2 * EO + n];
-                        const uint4 x = xb[4 * n - 8 * c - i];
-#pragma unroll
-                        for (int s = 0; s < 4; ++s) {
-                            l2[s] = dp2a<true, false>(e.x, word_of(x, s), l2[s]);
-                            l2[s] = dp2a<true, true>(e.y, word_of(x, s), l2[s]);
-                        }
-                    }
-#pragma unroll
-                    for (int s = 0; s < 4; ++s) g[c][s] += (int64_t)l2[s] << 32;
-                }
-            }
-            bool apply = true;
-            if constexpr (PER) {
-                apply = ++in_period == prm.period || (last_batch && bb + 1 == nb);
-                if (apply) in_period = 0;
-#pragma unroll
-                for (int c = 0; c < 2; ++c)
-#pragma unroll
-                    for (int s = 0; s < 4; ++s) g[c][s] = acc[c][s] += g[c][s];
-            }
-            if (apply) {
+            if (!PER && !any && !wide) {
+                // the common case in 32 bits
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
 #pragma unroll
                     for (int s = 0; s < 4; ++s) {
-                        T[c][s] = add_tap(T[c][s], g[c][s] >> mu);
+                        T[c][s] = add_tap32(T[c][s], l1[c][s], l0[c][s], mu);
                         wrow[tap_slot(s, i + 8 * c)] = (int16_t)(T[c][s] >> 16);
-                        if (PER) acc[c][s] = 0;
                     }
+            } else {
+                bool apply = true;
+                if constexpr (PER) {
+                    apply = ++in_period == prm.period || (last_batch && bb + 1 == nb);
+                    if (apply) in_period = 0;
+                }
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    int32_t l2[4] = {0, 0, 0, 0};
+                    if (any) {
+                        for (int n = 0; n < NG; ++n) {
+                            const uint2 e = s_ez2[S2 * EO + n];
+                            const uint4 x = xb[4 * n - 8 * c - i];
+#pragma unroll
+                            for (int s = 0; s < 4; ++s) {
+                                l2[s] = dp2a<true, false>(e.x, word_of(x, s), l2[s]);
+                                l2[s] = dp2a<true, true>(e.y, word_of(x, s), l2[s]);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) {
+                        int64_t g = (int64_t)l1[c][s] * 65536 + l0[c][s] + ((int64_t)l2[s] << 32);
+                        if (PER) g += acc[PER ? c : 0][s];
+                        if (apply) {
+                            T[c][s] = add_tap(T[c][s], g >> mu);
+                            wrow[tap_slot(s, i + 8 * c)] = (int16_t)(T[c][s] >> 16);
+                        }
+                        if (PER) acc[PER ? c : 0][s] = apply ? 0 : g;
+                    }
+                }
+                if (apply) wide = false;
             }
             __syncwarp();                          // taps published, limbs free
         }
@@ -501,9 +572,9 @@ void launch_na(bool split, const DevFrame *frames, const AeqChain *chains, int n
                cudaStream_t stream) {
     const unsigned n = (unsigned)n_chains;
     if (split && prm.period > 1)
-        aeq_split_kernel<NA, true><<<2 * n, 160, 0, stream>>>(frames, chains, prm);
+        aeq_split_kernel<NA, true><<<2 * n, SplitCfg<NA>::NT, 0, stream>>>(frames, chains, prm);
     else if (split)
-        aeq_split_kernel<NA, false><<<2 * n, 160, 0, stream>>>(frames, chains, prm);
+        aeq_split_kernel<NA, false><<<2 * n, SplitCfg<NA>::NT, 0, stream>>>(frames, chains, prm);
     else if (prm.period > 1)
         aeq_pair_kernel<NA, true><<<n, 32, 0, stream>>>(frames, chains, prm);
     else

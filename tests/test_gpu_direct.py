@@ -119,3 +119,20 @@ def test_aeq_freq_sum_plans(orc, fs):
     torch.cuda.synchronize()
     ref, Tr = orc.aeq(x, T0, 32, 2, mu_shift=12, rde_a=64, freq_sum=fs)
     assert np.array_equal(out.cpu().numpy(), ref) and np.array_equal(st.cpu().numpy(), Tr)
+
+
+@pytest.mark.parametrize("copies", [1, 700])
+@pytest.mark.parametrize("na,alpha", [(32, 2), (64, 4080)])
+def test_aeq_state_beyond_range(orc, na, alpha, copies):
+    """A state beyond the 30-bit range (inputs small enough that no transform
+    wraps) is used as it is and clamped by the first update."""
+    rng = np.random.default_rng(na + copies)
+    x = rng.integers(-2, 3, (300, 4)).astype(np.int8)
+    T0 = rng.integers(-(1 << 30), 1 << 30, (4, 4, 16)).astype(np.int32)
+    plan = F.Plan(n_aeq=na, alpha_aeq=alpha, mu_shift=9)
+    xd, out = dev(x), poison((copies, 300, 4))
+    st = dev(np.stack([T0] * copies))
+    F.aeq_run(plan, [F.Frame(xd, o, state=s) for o, s in zip(out, st)])
+    torch.cuda.synchronize()
+    ref, Tr = orc.aeq(x, T0, na, alpha, mu_shift=9, rde_a=64)
+    assert (out.cpu().numpy() == ref).all() and (st.cpu().numpy() == Tr).all()
