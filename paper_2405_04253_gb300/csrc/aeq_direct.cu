@@ -28,8 +28,8 @@
 // blocks is transposed at once while the next batch's words arrive by cp.async.
 //
 // Two layouts; aeq_direct_launch picks one (rule and figures there).
-//   aeq_pair_kernel   a warp per chain, both polarisations: many chains, bound by
-//                     dp2a issue and shared-memory loads
+//   aeq_duo_kernel    a warp per (chain, polarisation): many chains, bound by dp2a issue
+//                     and shared-memory loads
 //   aeq_split_kernel  six or eight warps per (chain, polarisation), by role: few
 //                     chains, bound by the latency of one block
 #include <algorithm>
@@ -110,8 +110,8 @@ __device__ __forceinline__ int32_t add_tap32(int32_t T, int32_t l1, int32_t l0, 
 
 __device__ __forceinline__ bool tap_in_range(int32_t T) { return T >= -(1 << 29) && T < (1 << 29); }
 
-// A warp's copies of symbols tb - K + q, q < XW (zero outside [lo, end)), to xn.
-template <class C>
+// Copies of symbols tb - K + q, q < XW (zero outside [lo, end)), to xn, by NTHR threads.
+template <class C, int NTHR = 32>
 __device__ __forceinline__ void stage(uint32_t *xn, const uint32_t *xin, int64_t tb, int64_t lo, int64_t end,
                                       int lane) {
     const int64_t t0 = tb - C::K;
@@ -120,31 +120,31 @@ __device__ __forceinline__ void stage(uint32_t *xn, const uint32_t *xin, int64_t
     const int q0 = (int)min(max(lo - t0, (int64_t)0), (int64_t)C::XW);
     const int q1 = (int)min(max(end - t0, (int64_t)0), (int64_t)C::XW);
 #pragma unroll
-    for (int q = lane; q < (C::XW + 31) / 32 * 32; q += 32) {
+    for (int q = lane; q < (C::XW + NTHR - 1) / NTHR * NTHR; q += NTHR) {
         if (q >= C::XW) break;
         const bool ok = q >= q0 && q < q1;
         cp_async4(xn + q, ok ? src + q : xin, ok);
     }
 }
 
-// xq[q] <- the byte transpose of the staged words q .. q + 3, by one warp, four
-// words of q a lane at a time (loads before stores).
-template <class C>
+// xq[q] <- the byte transpose of the staged words q .. q + 3, by NTHR threads, four
+// words of q a thread at a time (loads before stores).
+template <class C, int NTHR = 32>
 __device__ __forceinline__ void transpose(const uint32_t *xn, uint4 *xq, int lane) {
     constexpr int NQ = C::XW - 3;
 #pragma unroll
-    for (int q0 = 0; q0 < NQ; q0 += 128) {
+    for (int q0 = 0; q0 < NQ; q0 += 4 * NTHR) {
         uint32_t w[4][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) w[j][c] = q0 + 32 * j < NQ ? xn[min(q0 + 32 * j + lane, NQ - 1) + c] : 0;
+            for (int c = 0; c < 4; ++c) w[j][c] = q0 + NTHR * j < NQ ? xn[min(q0 + NTHR * j + lane, NQ - 1) + c] : 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int q = q0 + 32 * j + lane;
+            const int q = q0 + NTHR * j + lane;
             const uint32_t ab0 = __byte_perm(w[j][0], w[j][1], 0x5140), ab1 = __byte_perm(w[j][0], w[j][1], 0x7362);
             const uint32_t cd0 = __byte_perm(w[j][2], w[j][3], 0x5140), cd1 = __byte_perm(w[j][2], w[j][3], 0x7362);
-            if (q0 + 32 * j < NQ && q < NQ)
+            if (q0 + NTHR * j < NQ && q < NQ)
                 xq[q] = make_uint4(__byte_perm(ab0, cd0, 0x5410), __byte_perm(ab0, cd0, 0x7632),
                                    __byte_perm(ab1, cd1, 0x5410), __byte_perm(ab1, cd1, 0x7632));
         }
@@ -212,16 +212,19 @@ __device__ __forceinline__ int32_t out_of(int32_t y) { return min(max(y >> 7, -3
 //
 // One CTA per (chain, polarisation), its warps by role, so that only what the next
 // step waits for lies between two of them:
-//   NC = SA / 16 output warps: lane = 16 o + i, output o, symbol i of the warp's 16
+//   NC = SA / 16 output warps: lane = 2 i + o, output o, symbol i of the warp's 16
 //     (no reduction), the error and the limbs of e z; between blocks they store the
 //     outputs and load the next block's symbols
-//   4 gradient warps, one per input s1: lane = 16 o + k, the gradient of one tap over
+//   4 gradient warps, one per input s1: lane = 2 k + o, the gradient of one tap over
 //     the block and its update; between blocks they load the next block's symbols
 //   1 staging warp: the next batch into the other half of xq, once a batch
-// Limbs go from output to gradient warps at barrier 1, taps back at barrier 3 (the
-// writers arrive, the readers wait); barrier 2 joins all warps once a batch.
-// What a block takes is the latency of that round trip: about 200 instructions a warp
-// at 3 to 4 cycles each when one warp held a whole block.
+// Limbs go from output to gradient warps at barrier 1, which also tells whether any
+// e z needs its third limb, taps back at barrier 3 (the writers arrive, the readers
+// wait); barrier 2 joins all warps once a batch.
+// What a block takes is the latency of that round trip: 0.24 us at N = 32 and 0.35 us
+// at N = 64 for a lone chain (0.60 and 0.83 us with the transforms on a CTA); with a
+// whole block in one warp it was 0.34 and 0.61 us, about 200 and 500 dependent
+// instructions at 3 to 4 cycles each.
 template <int NA>
 struct SplitCfg {
     static constexpr int NC = (NA - kAeqK) / 16;          // output warps
@@ -233,6 +236,18 @@ struct SplitCfg {
 template <int ID, int N>
 __device__ __forceinline__ void bar_arrive() {
     asm volatile("bar.arrive %0, %1;\n" ::"n"(ID), "n"(N) : "memory");
+}
+
+// Barrier that returns whether v was true in any of its threads.
+template <int ID, int N>
+__device__ __forceinline__ bool bar_or(bool v) {
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"((uint32_t)v), "n"(ID), "n"(N)
+        : "memory");
+    return r != 0;
 }
 
 template <int NA, bool PER>
@@ -248,7 +263,6 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
     __shared__ uint4 s_w[2 * WO];
     __shared__ uint4 s_ez[2 * NG];
     __shared__ uint2 s_ez2[2 * NG];
-    __shared__ uint4 s_big;                       // word w: output warp w stored third limbs
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -259,11 +273,10 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
     const int64_t nblk = (ch.end - ch.begin + SA - 1) / SA;
     const int64_t nbatch = (nblk + C::PB - 1) / C::PB;
     const int mu = prm.mu_shift;
-    const int o = lane >> 4, i = lane & 15;
+    const int o = lane & 1, i = lane >> 1;
 
     if (warp == NC + R::NGW) {
         // ---- staging
-        if (lane == 0) s_big = make_uint4(0, 0, 0, 0);
         stage<C>(s_xn, xin, ch.begin, ch.lo, ch.end, lane);
         for (int64_t j = 0; j < nbatch; ++j) {
             cp_async_wait_all();
@@ -300,14 +313,12 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
                 }
                 const int32_t z =
                     out_of(((y[0][0] + y[0][1]) + (y[1][0] + y[1][1])) + ((y[2][0] + y[2][1]) + (y[3][0] + y[3][1])));
-                const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 16);
+                const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 1);
                 if (mu < 63) {
                     const RdeLimbs v = rde_limbs(z, zp, A2, valid);
                     store_limbs(s_ez + o * NG, si, v);
-                    const bool any = __any_sync(0xffffffffu, v.c2 != 0);
-                    if (any) store_limb2(s_ez2 + o * NG, si, v);
-                    if (lane == 0) ((uint32_t *)&s_big)[warp] = any;
-                    bar_arrive<1, NCG>();          // limbs stored
+                    store_limb2(s_ez2 + o * NG, si, v);
+                    bar_or<1, NCG>(v.c2 != 0);     // limbs stored
                 }
                 xb += SA;
                 if (bb + 1 < nb) {
@@ -325,7 +336,8 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
         int16_t *wtap = (int16_t *)(s_w + o * WO) + tap_slot(s1, i);
         int32_t T = ch.init[((2 * p + o) * 4 + s1) * K + i];
         *wtap = (int16_t)(T >> 16);
-        bool wide = !tap_in_range(T);              // a caller's state, until the first update
+        // a caller's state may hold taps beyond the 30-bit range until the first update
+        bool wide = __any_sync(0xffffffffu, !tap_in_range(T));
         int64_t acc = 0;
         int in_period = 0;
         const uint4 *er = s_ez + o * NG;
@@ -338,12 +350,10 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
                 uint32_t x[NG];
 #pragma unroll
                 for (int n = 0; n < NG; ++n) x[n] = xs[16 * n];
-                bar_sync<1, NCG>();                // limbs stored
+                const bool any = bar_or<1, NCG>(false);   // limbs stored; some c2 is not 0
                 int32_t l0[4] = {0, 0, 0, 0}, l1[4] = {0, 0, 0, 0};
 #pragma unroll
                 for (int n = 0; n < NG; ++n) grad4(er[n], x[n], l0[n & 3], l1[n & 3]);
-                const uint4 big = s_big;
-                const bool any = NC == 1 ? big.x != 0 : (big.x | big.y | big.z) != 0;
                 const int32_t g0 = (l0[0] + l0[1]) + (l0[2] + l0[3]), g1 = (l1[0] + l1[1]) + (l1[2] + l1[3]);
                 if (!PER && !any && !wide) {
                     T = add_tap32(T, g1, g0, mu);
@@ -354,7 +364,6 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
                         int32_t l2 = 0;
 #pragma unroll
                         for (int n = 0; n < NG; ++n) {
-                            if (word_of(big, n / 4) == 0) continue;   // that warp's are all 0, not stored
                             const uint2 e = s_ez2[o * NG + n];
                             l2 = dp2a<true, false>(e.x, x[n], l2);
                             l2 = dp2a<true, true>(e.y, x[n], l2);
@@ -374,7 +383,6 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
                         wide = false;
                     }
                 }
-                __syncwarp();
                 bar_arrive<3, NCG>();              // taps published, limbs read
             }
         }
@@ -384,186 +392,157 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
 
 // ----------------------------------------------------------- many chains ----
 //
-// A warp per chain, both polarisations: lane = 8 S2 + i.  The lane forms symbols i,
-// i + 8, ... of output S2, then the gradient of taps i and i + 8 of S2 and all four
-// inputs over the block, and updates those eight taps.  Outputs and taps 8 apart
-// read the same staged words (4 apart by tap group), so a block of both
-// polarisations loads SA / 4 + 2 of them for each half of the work instead of SA / 4
-// and four per polarisation, group of 16 symbols and half: shared-memory loads
-// (two to four cycles each and SM) are what bounded a warp per (chain, polarisation).
+// A CTA of two warps per chain, a warp per polarisation that holds a whole block:
+// lane = 2 i + o forms symbols i, i + 16, ... of output o, then the gradient of tap i
+// of o and all four inputs over the block, and updates those four taps, so nothing is
+// reduced over lanes and two __syncwarp order a block.  The warps share the staged
+// batch and meet twice a batch.  Lanes 2 i and 2 i + 1 read the same staged word, so a
+// 16-byte load of the warp is two passes over shared memory, not four.  Bound by issue
+// once four warps share a scheduler: 0.73 us a block for 1,216 chains at N = 32, 1.64
+// us at N = 64.  (One warp for both polarisations shares more loads, but took 0.73 and
+// 1.65 us there and 0.49 to 0.73 us where this one takes 0.45 to 0.58.)
 template <int NA, bool PER>
-__global__ void __launch_bounds__(32) aeq_pair_kernel(const DevFrame *__restrict__ frames,
-                                                      const AeqChain *__restrict__ chains, AeqParams prm) {
+__global__ void __launch_bounds__(64) aeq_duo_kernel(const DevFrame *__restrict__ frames,
+                                                     const AeqChain *__restrict__ chains, AeqParams prm) {
     using C = DirCfg<NA>;
-    constexpr int K = C::K, SA = C::SA, NG = C::NG, M = SA / 8;
-    constexpr int WO = 10;                        // 16-byte words per tap row: rows 8 banks apart
-    constexpr int EO = NG + 2;                    // ... per limb row: rows 24 banks apart
+    constexpr int K = C::K, SA = C::SA, NG = C::NG, M = SA / 16;
+    constexpr int WO = 12;
     __shared__ uint4 s_xq[C::XW];
     __shared__ uint32_t s_xn[C::XW];
-    __shared__ uint4 s_w[4 * WO];
-    __shared__ uint4 s_ez[4 * EO];
-    __shared__ uint2 s_ez2[4 * EO];
+    __shared__ uint4 s_w[2][2 * WO];
+    __shared__ uint4 s_ez[2][2 * NG];
+    __shared__ uint2 s_ez2[2][2 * NG];
 
-    const int lane = threadIdx.x;
-    const int S2 = lane >> 3, i = lane & 7;
+    const int tid = threadIdx.x, lane = tid & 31, p = tid >> 5;
+    const int o = lane & 1, i = lane >> 1;
     const uint32_t A2 = (uint32_t)prm.rde_a * (uint32_t)prm.rde_a;
     const int mu = prm.mu_shift;
     const AeqChain ch = chains[blockIdx.x];
     const DevFrame &fr = frames[ch.frame];
     const uint32_t *xin = (const uint32_t *)fr.aeq_in;
 
-    int16_t *wrow = (int16_t *)(s_w + S2 * WO);
-    int32_t T[2][4];
-    int64_t acc[PER ? 2 : 1][4];
+    int16_t *wrow = (int16_t *)(s_w[p] + o * WO);
+    uint4 *ez = s_ez[p] + o * NG;
+    uint2 *ez2 = s_ez2[p] + o * NG;
+    int32_t T[4];
+    int64_t acc[4];
     bool wide = false;   // a caller's state may hold taps beyond the 30-bit range until the first update
 #pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            T[c][s] = ch.init[(S2 * 4 + s) * K + i + 8 * c];
-            wide |= !tap_in_range(T[c][s]);
-            wrow[tap_slot(s, i + 8 * c)] = (int16_t)(T[c][s] >> 16);
-            if (PER) acc[c][s] = 0;
-        }
-
+    for (int s = 0; s < 4; ++s) {
+        T[s] = ch.init[((2 * p + o) * 4 + s) * K + i];
+        wide |= !tap_in_range(T[s]);
+        wrow[tap_slot(s, i)] = (int16_t)(T[s] >> 16);
+        acc[s] = 0;
+    }
     wide = __any_sync(0xffffffffu, wide);
-
     const int64_t nblk = (ch.end - ch.begin + SA - 1) / SA;
-    stage<C>(s_xn, xin, ch.begin, ch.lo, ch.end, lane);
+    stage<C, 64>(s_xn, xin, ch.begin, ch.lo, ch.end, tid);
     int in_period = 0;
     for (int64_t b0 = 0; b0 < nblk; b0 += C::PB) {
         const int64_t tb = ch.begin + b0 * SA;
         cp_async_wait_all();
-        __syncwarp();
-        transpose<C>(s_xn, s_xq, lane);
-        __syncwarp();
-        if (b0 + C::PB < nblk) stage<C>(s_xn, xin, tb + C::B, ch.lo, ch.end, lane);
+        __syncthreads();
+        transpose<C, 64>(s_xn, s_xq, tid);
+        __syncthreads();
+        if (b0 + C::PB < nblk) stage<C, 64>(s_xn, xin, tb + C::B, ch.lo, ch.end, tid);
         const int nb = (int)min((int64_t)C::PB, nblk - b0);
         const bool last_batch = b0 + C::PB >= nblk;
-        // valid and kept symbols relative to the batch
         const int rel_end = (int)min(ch.end - tb, (int64_t)C::B);
         const int rel_keep = (int)min(max(ch.keep - tb, (int64_t)0), (int64_t)C::B);
-        int16_t *outb = (int16_t *)fr.out + tb * 4 + (S2 & 2);
+        int16_t *outb = (int16_t *)fr.out + tb * 4 + 2 * p;
         for (int bb = 0; bb < nb; ++bb) {
             const uint4 *xb = s_xq + K + bb * SA;
-
-            // ---- convolution: symbol i + 8 m, tap group kg read word i - 15 + 4 (2 m + 3 - kg)
+            // ---- convolution, outputs, RDE error, limbs of e z
             int32_t y0[M], y1[M];
-            {
-                const uint4 *wr = s_w + S2 * WO;
-                uint4 wa[4], wb[4];
+            const uint4 *wr = s_w[p] + o * WO;
 #pragma unroll
-                for (int kg = 0; kg < 4; ++kg) {
-                    wa[kg] = wr[kg];
-                    wb[kg] = wr[4 + kg];
-                }
+            for (int m = 0; m < M; ++m) y0[m] = y1[m] = 0;
 #pragma unroll
-                for (int m = 0; m < M; ++m) y0[m] = y1[m] = 0;
+            for (int kg = 0; kg < 4; ++kg) {
+                const uint4 wa = wr[kg], wb = wr[4 + kg];
 #pragma unroll
-                for (int j = 0; j < 2 * M + 2; ++j) {
-                    const uint4 x = xb[i - 15 + 4 * j];
-#pragma unroll
-                    for (int m = 0; m < M; ++m) {
-                        const int kg = 2 * m + 3 - j;
-                        if (kg >= 0 && kg < 4) conv4(wa[kg & 3], wb[kg & 3], x, y0[m], y1[m]);
-                    }
-                }
+                for (int m = 0; m < M; ++m) conv4(wa, wb, xb[16 * m + i - 4 * kg - 3], y0[m], y1[m]);
             }
-
-            // ---- outputs, RDE error, limbs of e z
             bool big = false;
             RdeLimbs v[M];
 #pragma unroll
             for (int m = 0; m < M; ++m) {
-                const int si = i + 8 * m, rel = bb * SA + si;
+                const int si = i + 16 * m, rel = bb * SA + si;
                 const int32_t z = out_of(y0[m] + y1[m]);
-                const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 8);
+                const int32_t zp = __shfl_xor_sync(0xffffffffu, z, 1);
                 const bool valid = rel < rel_end;
                 v[m] = rde_limbs(z, zp, A2, valid);
-                store_limbs(s_ez + S2 * EO, si, v[m]);
+                store_limbs(ez, si, v[m]);
                 big |= v[m].c2 != 0;
-                if (valid && rel >= rel_keep && (S2 & 1) == 0)
+                if (valid && rel >= rel_keep && o == 0)
                     *(uint32_t *)(outb + rel * 4) = ((uint32_t)z & 0xFFFFu) | ((uint32_t)zp << 16);
             }
             const bool any = __any_sync(0xffffffffu, big);
             if (any) {
 #pragma unroll
-                for (int m = 0; m < M; ++m) store_limb2(s_ez2 + S2 * EO, i + 8 * m, v[m]);
+                for (int m = 0; m < M; ++m) store_limb2(ez2, i + 16 * m, v[m]);
             }
             __syncwarp();
             if (mu >= 63) continue;                // the taps never move: no gradient
 
-            // ---- gradient of eq. (6): tap i + 8 c, symbol group n read word
-            // -i - 8 + 4 (n - 2 c + 2)
-            int32_t l0[2][4], l1[2][4];
+            // ---- gradient of eq. (6) and update
+            int32_t l0[4], l1[4];
 #pragma unroll
-            for (int c = 0; c < 2; ++c)
+            for (int s = 0; s < 4; ++s) l0[s] = l1[s] = 0;
 #pragma unroll
-                for (int s = 0; s < 4; ++s) l0[c][s] = l1[c][s] = 0;
-            const uint4 *er = s_ez + S2 * EO;
-            uint4 e0 = er[0], e1 = er[0], e2;      // limbs of groups j, j - 1, j - 2
+            for (int n = 0; n < NG; ++n) {
+                const uint4 e = ez[n], x = xb[4 * n - i];
 #pragma unroll
-            for (int j = 0; j < NG + 2; ++j) {
-                e2 = e1;
-                e1 = e0;
-                if (j < NG) e0 = er[j];
-                const uint4 x = xb[4 * j - 8 - i];
-#pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    if (j >= 2) grad4(e2, word_of(x, s), l0[0][s], l1[0][s]);
-                    if (j < NG) grad4(e0, word_of(x, s), l0[1][s], l1[1][s]);
-                }
+                for (int s = 0; s < 4; ++s) grad4(e, word_of(x, s), l0[s], l1[s]);
             }
             if (!PER && !any && !wide) {
-                // the common case in 32 bits
 #pragma unroll
-                for (int c = 0; c < 2; ++c)
-#pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        T[c][s] = add_tap32(T[c][s], l1[c][s], l0[c][s], mu);
-                        wrow[tap_slot(s, i + 8 * c)] = (int16_t)(T[c][s] >> 16);
-                    }
+                for (int s = 0; s < 4; ++s) {
+                    T[s] = add_tap32(T[s], l1[s], l0[s], mu);
+                    wrow[tap_slot(s, i)] = (int16_t)(T[s] >> 16);
+                }
             } else {
+                int64_t g[4];
+#pragma unroll
+                for (int s = 0; s < 4; ++s) g[s] = (PER ? acc[s] : 0) + (int64_t)l1[s] * 65536 + l0[s];
+                if (any) {
+                    int32_t l2[4] = {0, 0, 0, 0};
+                    for (int n = 0; n < NG; ++n) {
+                        const uint2 e = ez2[n];
+                        const uint4 x = xb[4 * n - i];
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) {
+                            l2[s] = dp2a<true, false>(e.x, word_of(x, s), l2[s]);
+                            l2[s] = dp2a<true, true>(e.y, word_of(x, s), l2[s]);
+                        }
+                    }
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) g[s] += (int64_t)l2[s] << 32;
+                }
                 bool apply = true;
                 if constexpr (PER) {
                     apply = ++in_period == prm.period || (last_batch && bb + 1 == nb);
                     if (apply) in_period = 0;
                 }
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    int32_t l2[4] = {0, 0, 0, 0};
-                    if (any) {
-                        for (int n = 0; n < NG; ++n) {
-                            const uint2 e = s_ez2[S2 * EO + n];
-                            const uint4 x = xb[4 * n - 8 * c - i];
-#pragma unroll
-                            for (int s = 0; s < 4; ++s) {
-                                l2[s] = dp2a<true, false>(e.x, word_of(x, s), l2[s]);
-                                l2[s] = dp2a<true, true>(e.y, word_of(x, s), l2[s]);
-                            }
-                        }
-                    }
+                if (apply) {
 #pragma unroll
                     for (int s = 0; s < 4; ++s) {
-                        int64_t g = (int64_t)l1[c][s] * 65536 + l0[c][s] + ((int64_t)l2[s] << 32);
-                        if (PER) g += acc[PER ? c : 0][s];
-                        if (apply) {
-                            T[c][s] = add_tap(T[c][s], g >> mu);
-                            wrow[tap_slot(s, i + 8 * c)] = (int16_t)(T[c][s] >> 16);
-                        }
-                        if (PER) acc[PER ? c : 0][s] = apply ? 0 : g;
+                        T[s] = add_tap(T[s], g[s] >> mu);
+                        wrow[tap_slot(s, i)] = (int16_t)(T[s] >> 16);
                     }
+                    wide = false;
                 }
-                if (apply) wide = false;
+                if constexpr (PER) {
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) acc[s] = apply ? 0 : g[s];
+                }
             }
             __syncwarp();                          // taps published, limbs free
         }
     }
     if (ch.write_state) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int s = 0; s < 4; ++s) fr.state[(S2 * 4 + s) * K + i + 8 * c] = T[c][s];
+        for (int s = 0; s < 4; ++s) fr.state[((2 * p + o) * 4 + s) * K + i] = T[s];
     }
 }
 
@@ -576,22 +555,26 @@ void launch_na(bool split, const DevFrame *frames, const AeqChain *chains, int n
     else if (split)
         aeq_split_kernel<NA, false><<<2 * n, SplitCfg<NA>::NT, 0, stream>>>(frames, chains, prm);
     else if (prm.period > 1)
-        aeq_pair_kernel<NA, true><<<n, 32, 0, stream>>>(frames, chains, prm);
+        aeq_duo_kernel<NA, true><<<n, 64, 0, stream>>>(frames, chains, prm);
     else
-        aeq_pair_kernel<NA, false><<<n, 32, 0, stream>>>(frames, chains, prm);
+        aeq_duo_kernel<NA, false><<<n, 64, 0, stream>>>(frames, chains, prm);
 }
 
 }  // namespace
 
-// The split layout takes fewer cycles a block while the GPU is not full; the pair
-// layout fewer cycles of an SM a block.  total / longest is how many chains of the
-// longest one's length the launch amounts to.
+// The split layout takes fewer cycles a block while the GPU is not full, the duo layout
+// fewer cycles of an SM a block.  total / longest is how many chains of the longest
+// one's length the launch amounts to.  Measured with equal chains, us a block (split,
+// duo), by (chain, polarisation) items per SM (152 SMs):
+//            1            2            3            4            5            6
+//   N = 64   .352  .621   .466  .628   .601  .628   .749  .634   1.00  .914   1.13  .913
+//   N = 32   .243  .339   .260  .340   .317  .345   .354  .346   .429  .444   .622  .444
 cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
                               int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
                               cudaStream_t stream) {
     if (n_chains <= 0) return cudaSuccess;
     const double items = 2.0 * (double)total_symbols / (double)std::max<int64_t>(longest_symbols, 1);
-    const bool split = items < (na == 64 ? 5.0 : 7.0) * n_sm;
+    const bool split = items < (na == 64 ? 3.2 : 4.0) * n_sm;
     if (na == 64)
         launch_na<64>(split, frames, chains, n_chains, prm, stream);
     else
