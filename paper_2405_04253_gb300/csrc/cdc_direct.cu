@@ -17,8 +17,13 @@
 // Stores are 16 bytes (chain) or, where the buffer is 32-byte aligned, 32 bytes a
 // lane (CDC).
 //
-// Bound: dp4a issue (36 a PDM sample at L = 17 against 12 bytes moved, about equal
-// to the HBM time) for the CDC, latency for small frames.
+// The polarisations run one after the other (56 registers, 36 warps an SM; both at
+// once took 80 registers and 65.5 us) with the tap loop unrolled, so no register moves
+// between tap groups.
+//
+// Bound: dp4a issue (40 a PDM sample at L = 19 against 12 bytes moved, about equal to
+// the HBM time) for the CDC: 2^24 PDM samples, 19 taps in 53 us, 3.8 TB/s (245 us with
+// the transforms).  Latency for small frames.
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -114,60 +119,61 @@ __device__ __forceinline__ void cdc_tile(const DevFrame &fr, int64_t tile, uint3
         if (lane + 32 * it < NP) put(lane + 32 * it, a[it], b[it]);
     __syncwarp();
 
-    int32_t re[2][NPOL][4], im[2][NPOL][4];
-    uint4 cur[2][NPOL];                          // pw[u0 .. u0 + 3] of the chunk's first pair
+    // one polarisation after the other: res packs its 8 outputs (CDC: re, im as 16
+    // bits; chain: the two requantised bytes)
+    uint32_t res[NPOL][2][4];
+    [[maybe_unused]] const int sft = CHAIN ? fr.shift : 0;
+    [[maybe_unused]] const int32_t rnd = sft > 0 ? (1 << (sft - 1)) : 0;
 #pragma unroll
-    for (int g = 0; g < 2; ++g)
+    for (int p = 0; p < NPOL; ++p) {
+        int32_t re[2][4] = {}, im[2][4] = {};
+        uint4 cur[2];                            // pw[u0 .. u0 + 3] of the chunk's first pair
 #pragma unroll
-        for (int p = 0; p < NPOL; ++p) {
-            cur[g][p] = *(const uint4 *)(pw + C::base(g, p) + kHistPairs + 4 * lane);
+        for (int g = 0; g < 2; ++g) cur[g] = *(const uint4 *)(pw + C::base(g, p) + kHistPairs + 4 * lane);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) re[g][p][j] = im[g][p][j] = 0;
+        for (int c = 0; c < kHistPairs / 4; ++c) {
+            if (4 * c >= np) break;
+            const int4 h01 = *(const int4 *)(tw + 4 * c), h23 = *(const int4 *)(tw + 4 * c + 2);
+            uint32_t w[2][7];
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                const uint4 A = cur[g];
+                const uint4 B = *(const uint4 *)(pw + C::base(g, p) + kHistPairs - 4 + 4 * lane - 4 * c);
+                w[g][0] = B.y, w[g][1] = B.z, w[g][2] = B.w;
+                w[g][3] = A.x, w[g][4] = A.y, w[g][5] = A.z, w[g][6] = A.w;
+                cur[g] = B;
+            }
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                if (m > 0 && 4 * c + m >= np) break;
+                const int hr = m == 0 ? h01.x : m == 1 ? h01.z : m == 2 ? h23.x : h23.z;
+                const int hi = m == 0 ? h01.y : m == 1 ? h01.w : m == 2 ? h23.y : h23.w;
+#pragma unroll
+                for (int g = 0; g < 2; ++g)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        re[g][j] = __dp4a((int)w[g][3 + j - m], hr, re[g][j]);
+                        im[g][j] = __dp4a((int)w[g][3 + j - m], hi, im[g][j]);
+                    }
+            }
         }
-#pragma unroll 1
-    for (int c = 0; 4 * c < np; ++c) {
-        const int4 h01 = *(const int4 *)(tw + 4 * c), h23 = *(const int4 *)(tw + 4 * c + 2);
-        const int left = np - 4 * c;
 #pragma unroll
         for (int g = 0; g < 2; ++g)
 #pragma unroll
-            for (int p = 0; p < NPOL; ++p) {
-                const uint4 A = cur[g][p];
-                const uint4 B = *(const uint4 *)(pw + C::base(g, p) + kHistPairs - 4 + 4 * lane - 4 * c);
-                const uint32_t w[7] = {B.y, B.z, B.w, A.x, A.y, A.z, A.w};
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    if (m > 0 && m >= left) break;
-                    const int hr = m == 0 ? h01.x : m == 1 ? h01.z : m == 2 ? h23.x : h23.z;
-                    const int hi = m == 0 ? h01.y : m == 1 ? h01.w : m == 2 ? h23.y : h23.w;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        re[g][p][j] = __dp4a((int)w[3 + j - m], hr, re[g][p][j]);
-                        im[g][p][j] = __dp4a((int)w[3 + j - m], hi, im[g][p][j]);
-                    }
-                }
-                cur[g][p] = B;
-            }
+            for (int j = 0; j < 4; ++j)
+                res[p][g][j] = CHAIN ? __byte_perm((uint32_t)sat5((re[g][j] + rnd) >> sft),
+                                                   (uint32_t)sat5((im[g][j] + rnd) >> sft), 0x0040)
+                                     : __byte_perm((uint32_t)re[g][j], (uint32_t)im[g][j], 0x5410);
     }
 
     if constexpr (CHAIN) {
-        // requantise to 5 bits: symbols s0 + 128 g + 4 lane + j, a word (XI, XQ, YI, YQ) each
-        const int sft = fr.shift;
-        const int32_t rnd = sft > 0 ? (1 << (sft - 1)) : 0;
+        // symbols s0 + 128 g + 4 lane + j, a word (XI, XQ, YI, YQ) each
         uint32_t *dst = (uint32_t *)fr.aeq_in;
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
             uint32_t v[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                uint32_t b4[4];
-#pragma unroll
-                for (int p = 0; p < NPOL; ++p) {
-                    b4[2 * p] = (uint32_t)sat5((re[g][p][j] + rnd) >> sft);
-                    b4[2 * p + 1] = (uint32_t)sat5((im[g][p][j] + rnd) >> sft);
-                }
-                v[j] = __byte_perm(__byte_perm(b4[0], b4[1], 0x0040), __byte_perm(b4[2], b4[3], 0x0040), 0x5410);
-            }
+            for (int j = 0; j < 4; ++j) v[j] = __byte_perm(res[0][g][j], res[NPOL - 1][g][j], 0x5410);
             const int64_t s = tile * kTile + g * kHalf + 4 * lane;
             if (s + 4 <= fr.n_sym) {
                 *(uint4 *)(dst + s) = make_uint4(v[0], v[1], v[2], v[3]);
@@ -179,21 +185,20 @@ __device__ __forceinline__ void cdc_tile(const DevFrame &fr, int64_t tile, uint3
         }
     } else {
         // |z| <= 31 * 1024 fits 16 bits; samples t0 + 8 lane + 2 j + g
-        auto word = [&](int g, int p, int j) { return __byte_perm((uint32_t)re[g][p][j], (uint32_t)im[g][p][j], 0x5410); };
         uint32_t *dst = (uint32_t *)fr.out;
         const int64_t t = t0 + 8 * lane;
         if (t + 8 <= n && ((uintptr_t)dst & 31) == 0) {
             if constexpr (NPOL == 2) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const uint32_t v[8] = {word(0, 0, 2 * h), word(0, 1, 2 * h), word(1, 0, 2 * h), word(1, 1, 2 * h),
-                                           word(0, 0, 2 * h + 1), word(0, 1, 2 * h + 1), word(1, 0, 2 * h + 1),
-                                           word(1, 1, 2 * h + 1)};
+                    const uint32_t v[8] = {res[0][0][2 * h], res[1][0][2 * h], res[0][1][2 * h], res[1][1][2 * h],
+                                           res[0][0][2 * h + 1], res[1][0][2 * h + 1], res[0][1][2 * h + 1],
+                                           res[1][1][2 * h + 1]};
                     store32(dst + 2 * t + 8 * h, v);
                 }
             } else {
-                const uint32_t v[8] = {word(0, 0, 0), word(1, 0, 0), word(0, 0, 1), word(1, 0, 1),
-                                       word(0, 0, 2), word(1, 0, 2), word(0, 0, 3), word(1, 0, 3)};
+                const uint32_t v[8] = {res[0][0][0], res[0][1][0], res[0][0][1], res[0][1][1],
+                                       res[0][0][2], res[0][1][2], res[0][0][3], res[0][1][3]};
                 store32(dst + t, v);
             }
         } else {
@@ -203,9 +208,9 @@ __device__ __forceinline__ void cdc_tile(const DevFrame &fr, int64_t tile, uint3
                 for (int g = 0; g < 2; ++g) {
                     if (t + 2 * j + g >= n) continue;
                     if constexpr (NPOL == 2)
-                        *(uint2 *)(dst + 2 * (t + 2 * j + g)) = make_uint2(word(g, 0, j), word(g, 1, j));
+                        *(uint2 *)(dst + 2 * (t + 2 * j + g)) = make_uint2(res[0][g][j], res[1][g][j]);
                     else
-                        dst[t + 2 * j + g] = word(g, 0, j);
+                        dst[t + 2 * j + g] = res[0][g][j];
                 }
         }
     }
