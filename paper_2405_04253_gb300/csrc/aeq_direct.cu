@@ -253,7 +253,8 @@ __device__ __forceinline__ bool bar_or(bool v) {
 template <int NA, bool PER>
 __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFrame *__restrict__ frames,
                                                                      const AeqChain *__restrict__ chains,
-                                                                     AeqParams prm) {
+                                                                     AeqParams prm,
+                                                                     const __grid_constant__ SingleFrame one) {
     using C = DirCfg<NA>;
     using R = SplitCfg<NA>;
     constexpr int K = C::K, SA = C::SA, NG = C::NG, NC = R::NC, NCG = R::NCG;
@@ -266,10 +267,13 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const AeqChain ch = chains[blockIdx.x >> 1];
+    const AeqChain ch = chains ? chains[blockIdx.x >> 1] : single_chain(one, blockIdx.x >> 1);
     const int p = blockIdx.x & 1;
-    const DevFrame &fr = frames[ch.frame];
-    const uint32_t *xin = (const uint32_t *)fr.aeq_in;
+    const DevFrame &fr = chains ? frames[ch.frame] : one.fr;
+    // (read once: nothing may be kept over the barriers' memory clobbers)
+    const uint32_t *const xin = (const uint32_t *)fr.aeq_in;
+    int16_t *const out = (int16_t *)fr.out;
+    int32_t *const state = fr.state;
     const int64_t nblk = (ch.end - ch.begin + SA - 1) / SA;
     const int64_t nbatch = (nblk + C::PB - 1) / C::PB;
     const int mu = prm.mu_shift;
@@ -298,7 +302,7 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
             // valid and kept symbols relative to the batch, less the lane's
             const int left = (int)min(ch.end - tb, (int64_t)C::B) - si;
             const int skip = (int)min(max(ch.keep - tb, (int64_t)0), (int64_t)C::B) - si;
-            int16_t *dst = (int16_t *)fr.out + (tb + si) * 4 + 2 * p;
+            int16_t *dst = out + (tb + si) * 4 + 2 * p;
             const uint4 *xb = s_xq[j & 1] + K + si - 3;
             uint4 x[4];                           // a block ahead
 #pragma unroll
@@ -386,7 +390,7 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
                 bar_arrive<3, NCG>();              // taps published, limbs read
             }
         }
-        if (ch.write_state) fr.state[((2 * p + o) * 4 + s1) * K + i] = T;
+        if (ch.write_state) state[((2 * p + o) * 4 + s1) * K + i] = T;
     }
 }
 
@@ -403,7 +407,8 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
 // 1.65 us there and 0.49 to 0.73 us where this one takes 0.45 to 0.58.)
 template <int NA, bool PER>
 __global__ void __launch_bounds__(64) aeq_duo_kernel(const DevFrame *__restrict__ frames,
-                                                     const AeqChain *__restrict__ chains, AeqParams prm) {
+                                                     const AeqChain *__restrict__ chains, AeqParams prm,
+                                                     const __grid_constant__ SingleFrame one) {
     using C = DirCfg<NA>;
     constexpr int K = C::K, SA = C::SA, NG = C::NG, M = SA / 16;
     constexpr int WO = 12;
@@ -417,9 +422,11 @@ __global__ void __launch_bounds__(64) aeq_duo_kernel(const DevFrame *__restrict_
     const int o = lane & 1, i = lane >> 1;
     const uint32_t A2 = (uint32_t)prm.rde_a * (uint32_t)prm.rde_a;
     const int mu = prm.mu_shift;
-    const AeqChain ch = chains[blockIdx.x];
-    const DevFrame &fr = frames[ch.frame];
-    const uint32_t *xin = (const uint32_t *)fr.aeq_in;
+    const AeqChain ch = chains ? chains[blockIdx.x] : single_chain(one, blockIdx.x);
+    const DevFrame &fr = chains ? frames[ch.frame] : one.fr;
+    const uint32_t *const xin = (const uint32_t *)fr.aeq_in;
+    int16_t *const out = (int16_t *)fr.out;
+    int32_t *const state = fr.state;
 
     int16_t *wrow = (int16_t *)(s_w[p] + o * WO);
     uint4 *ez = s_ez[p] + o * NG;
@@ -449,7 +456,7 @@ __global__ void __launch_bounds__(64) aeq_duo_kernel(const DevFrame *__restrict_
         const bool last_batch = b0 + C::PB >= nblk;
         const int rel_end = (int)min(ch.end - tb, (int64_t)C::B);
         const int rel_keep = (int)min(max(ch.keep - tb, (int64_t)0), (int64_t)C::B);
-        int16_t *outb = (int16_t *)fr.out + tb * 4 + 2 * p;
+        int16_t *outb = out + tb * 4 + 2 * p;
         for (int bb = 0; bb < nb; ++bb) {
             const uint4 *xb = s_xq + K + bb * SA;
             // ---- convolution, outputs, RDE error, limbs of e z
@@ -542,23 +549,25 @@ __global__ void __launch_bounds__(64) aeq_duo_kernel(const DevFrame *__restrict_
     }
     if (ch.write_state) {
 #pragma unroll
-        for (int s = 0; s < 4; ++s) fr.state[((2 * p + o) * 4 + s) * K + i] = T[s];
+        for (int s = 0; s < 4; ++s) state[((2 * p + o) * 4 + s) * K + i] = T[s];
     }
 }
 
 template <int NA>
 void launch_na(bool split, const DevFrame *frames, const AeqChain *chains, int n_chains, AeqParams prm,
-               cudaStream_t stream) {
+               cudaStream_t stream, const SingleFrame &one) {
     const unsigned n = (unsigned)n_chains;
     if (split && prm.period > 1)
-        aeq_split_kernel<NA, true><<<2 * n, SplitCfg<NA>::NT, 0, stream>>>(frames, chains, prm);
+        aeq_split_kernel<NA, true><<<2 * n, SplitCfg<NA>::NT, 0, stream>>>(frames, chains, prm, one);
     else if (split)
-        aeq_split_kernel<NA, false><<<2 * n, SplitCfg<NA>::NT, 0, stream>>>(frames, chains, prm);
+        aeq_split_kernel<NA, false><<<2 * n, SplitCfg<NA>::NT, 0, stream>>>(frames, chains, prm, one);
     else if (prm.period > 1)
-        aeq_duo_kernel<NA, true><<<n, 64, 0, stream>>>(frames, chains, prm);
+        aeq_duo_kernel<NA, true><<<n, 64, 0, stream>>>(frames, chains, prm, one);
     else
-        aeq_duo_kernel<NA, false><<<n, 64, 0, stream>>>(frames, chains, prm);
+        aeq_duo_kernel<NA, false><<<n, 64, 0, stream>>>(frames, chains, prm, one);
 }
+
+const SingleFrame kNoSingle{};
 
 }  // namespace
 
@@ -571,14 +580,16 @@ void launch_na(bool split, const DevFrame *frames, const AeqChain *chains, int n
 //   N = 32   .243  .339   .260  .340   .317  .345   .354  .346   .429  .444   .622  .444
 cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
                               int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
-                              cudaStream_t stream) {
+                              cudaStream_t stream, const SingleFrame *one) {
     if (n_chains <= 0) return cudaSuccess;
+    const SingleFrame &single = one ? *one : kNoSingle;
+    if (one) frames = nullptr, chains = nullptr;
     const double items = 2.0 * (double)total_symbols / (double)std::max<int64_t>(longest_symbols, 1);
     const bool split = items < (na == 64 ? 3.2 : 4.0) * n_sm;
     if (na == 64)
-        launch_na<64>(split, frames, chains, n_chains, prm, stream);
+        launch_na<64>(split, frames, chains, n_chains, prm, stream, single);
     else
-        launch_na<32>(split, frames, chains, n_chains, prm, stream);
+        launch_na<32>(split, frames, chains, n_chains, prm, stream, single);
     return cudaGetLastError();
 }
 

@@ -332,11 +332,12 @@ bool fnt::aeq_use_serial(const fnt_plan *p, int64_t n_chains, int64_t longest_sy
 }
 
 cudaError_t fnt::aeq_launch_for(const fnt_plan *p, const DevFrame *frames, const AeqChain *chains, int n_chains,
-                                int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream) {
+                                int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream,
+                                const SingleFrame *one) {
     AeqParams prm{p->d.mu_shift, p->d.rde_a, update_period(p->d), p->tensor_gradient, p->d.aeq_freq_sum};
     if (aeq_use_direct(p))
         return aeq_direct_launch(p->d.n_aeq, frames, chains, n_chains, total_symbols, longest_symbols, prm, p->n_sm,
-                                 stream);
+                                 stream, one);
     if (aeq_use_serial(p, n_chains, longest_symbols))
         return aeq_serial_launch(p->d.n_aeq, frames, chains, n_chains, prm, 0, stream);
     return aeq_launch(p->d.n_aeq, frames, chains, n_chains, prm, p->aeq_warps, 0, stream, aeq_min_smem(p));
@@ -707,10 +708,17 @@ fnt_status upload_work(Work &w, char *dev, cudaStream_t stream) {
     return e == cudaSuccess ? FNT_OK : cuda_fail(e, "upload tables");
 }
 
+static SingleFrame work_single(const fnt_plan *p, const Work &w, const char *dev) {
+    const DevFrame &df = w.frames[0];
+    const int32_t *init = !w.init_src.empty() ? (const int32_t *)(dev + w.off_init) : df.state ? df.state : p->d_init;
+    return single_frame(p, df, init);
+}
+
 static fnt_status launch_cdc_range(const fnt_plan *p, const Work &w, const char *dev, int i0, int i1,
                                    cudaStream_t stream) {
     if (i1 <= i0) return FNT_OK;
     const DevFrame *frames = (const DevFrame *)(dev + w.off_frames);
+    if (w.single) return launch_single(p, work_single(p, w, dev), w.op, stream, 1);
     if (w.cdc_direct) {
         cudaError_t e = cdc_direct_launch(frames, (const int4 *)(dev + w.off_items) + i0, i1 - i0,
                                           w.op == FNT_OP_CHAIN, w.cdc_tiles, stream);
@@ -759,6 +767,8 @@ fnt_status launch_work(const fnt_plan *p, const Work &w, const char *dev, cudaSt
         st = launch_spectra(w, dev, stream);
         if (st == FNT_OK) st = launch_cdc_range(p, w, dev, 0, (int)w.items.size(), stream);
     }
+    if (st == FNT_OK && (stages & 2) && w.op != FNT_OP_CDC && w.single && aeq_use_direct(p))
+        return launch_single(p, work_single(p, w, dev), w.op, stream, 2);
     if (st == FNT_OK && (stages & 2) && w.op != FNT_OP_CDC && !w.chains.empty()) {
         st = copy_initial_taps(w, dev, stream);
         if (st == FNT_OK) st = launch_aeq_range(p, w, dev, 0, (int)w.chains.size(), stream);
@@ -790,6 +800,47 @@ fnt_status launch_pipelined(const fnt_plan *p, const Work &w, const char *dev, c
     return st;
 }
 
+bool single_direct(const fnt_plan *p, int op) {
+    return (op == FNT_OP_AEQ || cdc_use_direct(p)) && (op == FNT_OP_CDC || aeq_use_direct(p));
+}
+
+SingleFrame single_frame(const fnt_plan *p, const DevFrame &df, const int32_t *init) {
+    SingleFrame one{};
+    one.fr = df;
+    one.seg = p->d.aeq_segment > 0 && p->d.aeq_segment < df.n_sym ? p->d.aeq_segment : 0;
+    one.warmup = one.seg > 0 ? p->d.aeq_warmup : 0;
+    one.init = init;
+    return one;
+}
+
+int64_t single_chains(const SingleFrame &one) {
+    if (one.fr.n_sym == 0) return 0;
+    return one.seg > 0 ? (one.fr.n_sym + one.seg - 1) / one.seg : 1;
+}
+
+fnt_status launch_single(const fnt_plan *p, const SingleFrame &one, int op, cudaStream_t stream, int stages) {
+    cudaError_t e = cudaSuccess;
+    if ((stages & 1) && op != FNT_OP_AEQ) {
+        const int64_t tiles = cdc_direct_tiles(one.fr, op);
+        const int per = cdc_direct_tiles_per_item(p, tiles);
+        e = cdc_direct_launch(nullptr, nullptr, (int)((tiles + per - 1) / per), op == FNT_OP_CHAIN, per, stream, &one);
+        if (e != cudaSuccess) return cuda_fail(e, "direct cdc kernel launch");
+    }
+    const int64_t chains = op != FNT_OP_CDC ? single_chains(one) : 0;
+    if ((stages & 2) && chains > 0) {
+        if (one.seg > 0 && one.fr.state && one.init != one.fr.state) {
+            // segments start from the state as it was: the last one overwrites it
+            e = cudaMemcpyAsync((void *)one.init, one.fr.state, kStateBytes, cudaMemcpyDeviceToDevice, stream);
+            if (e != cudaSuccess) return cuda_fail(e, "copy initial taps");
+        }
+        const int64_t longest = one.seg > 0 ? std::min(one.fr.n_sym, one.seg + one.warmup) : one.fr.n_sym;
+        e = aeq_launch_for(p, nullptr, nullptr, (int)chains, one.fr.n_sym + (chains - 1) * one.warmup, longest, stream,
+                           &one);
+        if (e != cudaSuccess) return cuda_fail(e, "direct aeq kernel launch");
+    }
+    return FNT_OK;
+}
+
 int work_kernel_count(const Work &w) {
     const int C = (int)w.item_cut.size() - 1;
     int k = 0;
@@ -814,11 +865,69 @@ static size_t out_bytes(const fnt_frame &f, int op, const DevFrame &df) {
     return df.n_sym * 8;
 }
 
+// A call on one frame in direct form: no work tables, so nothing is built or uploaded,
+// and device memory is taken only for what the work itself needs (the chain's symbols,
+// a copy of the taps for segments, staging of pageable host buffers).
+static fnt_status run_single(const fnt_plan *p, const fnt_frame &f, int op, bool host, cudaStream_t stream) {
+    DevFrame df;
+    fnt_status st = make_frame(p, f, op, 0, df);
+    if (st != FNT_OK) return st;
+    const size_t nin = in_bytes(f, op), nout = out_bytes(f, op, df);
+    SingleFrame one = single_frame(p, df, df.state ? df.state : p->d_init);
+    if (single_chains(one) > INT32_MAX) return fail(FNT_ERR_INVALID, "batch too large");
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    size_t total = 0;
+    const size_t off_sym = total;
+    if (op == FNT_OP_CHAIN) total += up((size_t)df.n_sym * 4);
+    const size_t off_init = total;
+    const bool copy_init = op != FNT_OP_CDC && one.seg > 0 && df.state;
+    if (copy_init) total += up(kStateBytes);
+    void *vin = host && nin ? device_view(f.in) : nullptr, *vout = host && nout ? device_view(f.out) : nullptr;
+    const bool stage_in = host && nin && !vin, stage_out = host && nout && !vout;
+    const size_t off_in = total;
+    if (stage_in) total += up(nin);
+    const size_t off_out = total;
+    if (stage_out) total += up(nout);
+    char *dev = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (total > 0) {
+        e = cudaMallocFromPoolAsync((void **)&dev, total, p->pool, stream);
+        if (e != cudaSuccess)
+            return e == cudaErrorMemoryAllocation ? fail(FNT_ERR_NOMEM, "device memory")
+                                                  : cuda_fail(e, "cudaMallocFromPoolAsync");
+    }
+    DevFrame &fr = one.fr;
+    if (stage_in) vin = dev + off_in;
+    if (stage_out) vout = dev + off_out;
+    if (vin) fr.in = (const int8_t *)vin;
+    if (vout) fr.out = vout;
+    if (op == FNT_OP_AEQ) fr.aeq_in = (int8_t *)fr.in;
+    if (op == FNT_OP_CHAIN) fr.aeq_in = (int8_t *)(dev + off_sym);
+    if (copy_init) one.init = (const int32_t *)(dev + off_init);
+    if (stage_in) {
+        e = cudaMemcpyAsync(vin, f.in, nin, cudaMemcpyHostToDevice, stream);
+        if (e != cudaSuccess) st = cuda_fail(e, "copy input");
+    }
+    if (st == FNT_OK) st = launch_single(p, one, op, stream, 3);
+    if (st == FNT_OK && stage_out) {
+        e = cudaMemcpyAsync(f.out, vout, nout, cudaMemcpyDeviceToHost, stream);
+        if (e != cudaSuccess) st = cuda_fail(e, "copy output");
+    }
+    if (dev) cudaFreeAsync(dev, stream);
+    if (st == FNT_OK && host) {
+        e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) st = cuda_fail(e, "cudaStreamSynchronize");
+    }
+    return st;
+}
+
 static fnt_status run(const fnt_plan *p, const fnt_frame_batch *b, int op, void *stream_) {
     if (!p) return fail(FNT_ERR_INVALID, "null plan");
     fnt_status dst = check_device(p);
     if (dst != FNT_OK) return dst;
     cudaStream_t stream = (cudaStream_t)stream_;
+    if (b && b->n_frames == 1 && b->frames && single_direct(p, op))
+        return run_single(p, b->frames[0], op, b->host_buffers != 0, stream);
     Work w;
     fnt_status st = build_work(p, b, op, w);
     if (st != FNT_OK) return st;
@@ -980,6 +1089,8 @@ extern "C" fnt_status fnt_batch_create(const fnt_plan *p, const fnt_frame_batch 
     }
     layout(bt->work);
     const int C = (int)bt->work.item_cut.size() - 1;
+    // (host inputs may be repointed in the frame table after a graph is captured)
+    bt->work.single = bt->work.frames.size() == 1 && C == 1 && bt->inputs.empty() && single_direct(p, op);
     if (C > 1) {
         bt->side.resize(C);
         bt->ev.resize(2 * C);

@@ -218,29 +218,43 @@ __device__ __forceinline__ void cdc_tile(const DevFrame &fr, int64_t tile, uint3
 
 template <bool CHAIN>
 __global__ void __launch_bounds__(32 * kCdcDirectWarps) cdc_direct_kernel(const DevFrame *__restrict__ frames,
-                                                                          const int4 *__restrict__ items) {
+                                                                          const int4 *__restrict__ items,
+                                                                          const __grid_constant__ SingleFrame one) {
     __shared__ __align__(16) uint32_t s_pw[kCdcDirectWarps][CdcDirect<CHAIN, 2>::WORDS];
     __shared__ __align__(16) int2 s_tw[kCdcDirectWarps][kHistPairs];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int4 item = items[blockIdx.x];
-    if (warp >= item.z) return;
-    const DevFrame &fr = frames[item.x];
-    const int64_t tile = (int64_t)item.y + warp;
+    // (no tables for a single frame: they would cost two dependent loads, and a call
+    // their upload)
+    int64_t tile = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+    const DevFrame *pf = &one.fr;
+    if (items) {
+        const int4 item = items[blockIdx.x];
+        if (warp >= item.z) return;
+        pf = frames + item.x;
+        tile = (int64_t)item.y + warp;
+    } else if (tile * kTile >= (CHAIN ? one.fr.n_sym : one.fr.n)) {
+        return;
+    }
+    const DevFrame &fr = *pf;
     if (CHAIN || fr.n_pol == 2)
         cdc_tile<CHAIN, 2>(fr, tile, s_pw[warp], s_tw[warp], lane);
     else if constexpr (!CHAIN)
         cdc_tile<false, 1>(fr, tile, s_pw[warp], s_tw[warp], lane);
 }
 
+const SingleFrame kNoSingle{};
+
 }  // namespace
 
 cudaError_t cdc_direct_launch(const DevFrame *frames, const int4 *items, int n_items, bool chain, int warps,
-                              cudaStream_t stream) {
+                              cudaStream_t stream, const SingleFrame *one) {
     if (n_items <= 0) return cudaSuccess;
+    const SingleFrame &single = one ? *one : kNoSingle;
+    if (one) frames = nullptr, items = nullptr;
     if (chain)
-        cdc_direct_kernel<true><<<n_items, 32 * warps, 0, stream>>>(frames, items);
+        cdc_direct_kernel<true><<<n_items, 32 * warps, 0, stream>>>(frames, items, single);
     else
-        cdc_direct_kernel<false><<<n_items, 32 * warps, 0, stream>>>(frames, items);
+        cdc_direct_kernel<false><<<n_items, 32 * warps, 0, stream>>>(frames, items, single);
     return cudaGetLastError();
 }
 

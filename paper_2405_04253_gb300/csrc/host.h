@@ -55,6 +55,7 @@ struct Work {
     bool cdc_both = false;            // CDC items may cover both polarisations (item.w = 2)
     bool cdc_direct = false;          // CDC items are the direct kernel's (tiles of a frame)
     int cdc_tiles = 1;                // direct CDC: most tiles per item
+    bool single = false;              // one frame, taken by the direct kernels as a parameter
     bool spectra_ready = false;       // the frames' CDC tap spectra are computed (prepared batches)
     std::vector<DevFrame> frames;
     std::vector<int4> items;          // CDC: (frame, first block, blocks)
@@ -93,8 +94,9 @@ int work_kernel_count(const Work &w);
 constexpr int kCdcCtasPerSm = 3;     // cdc_kernel's __launch_bounds__ minimum
 constexpr int kSerialCtasPerSm = 1;  // aeq_serial_kernel CTAs resident per SM (registers)
 constexpr int kSerialMinBlocks = 256;  // shortest longest-chain (blocks) for which the automatic choice takes it
+// `one`: the work of a single frame, in place of the tables.
 cudaError_t cdc_direct_launch(const DevFrame *frames, const int4 *items, int n_items, bool chain, int warps,
-                              cudaStream_t stream);
+                              cudaStream_t stream, const SingleFrame *one = nullptr);
 size_t cdc_smem_bytes(int warps);
 int cdc_mults_per_block();
 int cdc_butterflies_per_block();
@@ -122,16 +124,24 @@ cudaError_t aeq_serial_launch(int na, const DevFrame *frames, const AeqChain *ch
 bool aeq_use_serial(const fnt_plan *p, int64_t n_chains, int64_t longest_symbols);
 // Launches the AEQ kernel the plan picks for those chains, of total_symbols in all.
 cudaError_t aeq_launch_for(const fnt_plan *p, const DevFrame *frames, const AeqChain *chains, int n_chains,
-                           int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream);
+                           int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream,
+                           const SingleFrame *one = nullptr);
 // The direct form of the AEQ (aeq_direct.cu).
 cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
                               int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
-                              cudaStream_t stream);
+                              cudaStream_t stream, const SingleFrame *one = nullptr);
 // Whether the plan's CDC and AEQ run in direct form (no transform kernel picked).
 bool cdc_use_direct(const fnt_plan *p);
 bool aeq_use_direct(const fnt_plan *p);
 // Tiles of a frame's direct CDC for `op`, and how many of `tiles` an item takes.
 int64_t cdc_direct_tiles(const DevFrame &df, int op);
 int cdc_direct_tiles_per_item(const fnt_plan *p, int64_t tiles);
+// Whether `op` on one frame runs in direct form throughout, so that its kernels take
+// the frame as a parameter; the AEQ runs of the frame then, from the taps at init; and
+// their launches (stages: bit 0 = CDC, bit 1 = AEQ).
+bool single_direct(const fnt_plan *p, int op);
+SingleFrame single_frame(const fnt_plan *p, const DevFrame &df, const int32_t *init);
+int64_t single_chains(const SingleFrame &one);
+fnt_status launch_single(const fnt_plan *p, const SingleFrame &one, int op, cudaStream_t stream, int stages);
 
 }  // namespace fnt

@@ -52,6 +52,15 @@ struct alignas(16) AeqChain {
 };
 static_assert(sizeof(AeqChain) == 64, "AeqChain layout");
 
+// The work of a call on one frame, as a kernel parameter instead of tables: CDC tiles
+// in order, and the AEQ runs of the frame by rule (runs of seg symbols, 0 for one run,
+// with warmup symbols before them, from the taps at init).
+struct SingleFrame {
+    DevFrame fr;
+    int64_t seg, warmup;
+    const int32_t *init;
+};
+
 struct AeqParams {
     int32_t mu_shift;
     int32_t rde_a;
@@ -61,6 +70,21 @@ struct AeqParams {
 };
 
 constexpr int kMaxUpdatePeriod = 64;   // keeps the summed int64 gradient exact
+
+#ifdef __CUDACC__
+// AEQ run c of a single frame (the table entries the host builds for many).
+__device__ __forceinline__ AeqChain single_chain(const SingleFrame &one, int64_t c) {
+    AeqChain ch{};
+    const int64_t n = one.fr.n_sym, k = c * one.seg;
+    ch.keep = k;
+    ch.end = one.seg > 0 && k + one.seg < n ? k + one.seg : n;
+    ch.begin = k > one.warmup ? k - one.warmup : 0;
+    ch.lo = ch.begin > kAeqK ? ch.begin - kAeqK : 0;
+    ch.write_state = one.fr.state != nullptr && ch.end == n;
+    ch.init = one.init;
+    return ch;
+}
+#endif
 
 // DevFrame::flags
 constexpr int32_t kFrameInjectTmaTimeout = 1;   // arm the CDC's window barrier without issuing its copy

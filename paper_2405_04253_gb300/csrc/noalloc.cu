@@ -145,6 +145,26 @@ extern "C" fnt_status fnt_cdc_aeq_run_noalloc(const fnt_plan *p, const fnt_frame
     char *base = g_dev_addr[dev];
     if (f->n == 0) return FNT_OK;
 
+    if (single_direct(p, FNT_OP_CHAIN)) {
+        // the direct kernels take the frame as a parameter: no tables
+        DevFrame df{};
+        df.in = (const int8_t *)f->in;
+        df.out = f->out;
+        df.aeq_in = (int8_t *)(base + kOffSym);
+        df.state = f->aeq_state;
+        df.n = f->n;
+        df.n_sym = nsym;
+        df.n_pol = 2;
+        df.L = f->cd_len;
+        df.S = S;
+        df.shift = cdc_shift_of(f->cd_taps, f->cd_len);
+        df.phase = phase;
+        memcpy(df.taps, f->cd_taps, 2 * (size_t)f->cd_len);
+        SingleFrame one = single_frame(p, df, f->aeq_state ? f->aeq_state : p->d_init);
+        if (one.seg > 0 && f->aeq_state) one.init = (const int32_t *)(base + kOffInit);
+        return launch_single(p, one, FNT_OP_CHAIN, stream, 3);
+    }
+
     const int mi = (int)(g_next++ % kMirrors);
     if (g_mirror_dev[mi] >= 0) {
         e = cudaEventSynchronize(g_mirror_done[mi][g_mirror_dev[mi]]);   // its last upload has run
