@@ -87,6 +87,23 @@ def aeq_ops(n_sym: int, na: int) -> float:
     return n_sym / sa * per_block
 
 
+# The direct forms do the convolutions that define the results: 8 operations a
+# complex tap and kept CDC output, 2 a real tap for the AEQ's convolutions and
+# again for its gradient (e z as one factor), at the rate of the instruction that
+# does them: dp4a four, dp2a two multiply-adds on 64 lanes a clock and SM.
+def cdc_direct_ops(n_out: int, L: int, n_pol: int = 2) -> float:
+    return 8.0 * n_out * n_pol * L
+
+
+def aeq_direct_ops(n_sym: int) -> float:
+    return 2.0 * 2 * 4 * 4 * 16 * n_sym
+
+
+def dot_peak_ops(products: int) -> float:
+    """Issue peak of dp4a (4 products) or dp2a (2): 152 SMs x 64 lanes x 2070 MHz."""
+    return 152 * 64 * 2 * products * 2070e6
+
+
 def alu_peak_ops() -> float:
     """Issue-bound INT32 peak: 152 SMs x 4 schedulers x 32 lanes x 2070 MHz."""
     return 152 * 4 * 32 * 2070e6
@@ -503,28 +520,40 @@ def run_fnt(args, rank, world, local_rank, oracle_pool=None):
     aeq_avg = statistics.mean(aeq_ms)
     cdc_avg = statistics.mean(cdc_ms)
     dom = "aeq" if aeq_avg >= cdc_avg else "cdc"
-    ops = aeq_ops(nsym, wl["n_aeq"]) if dom == "aeq" else cdc_ops(n, S)
     dur = aeq_avg if dom == "aeq" else cdc_avg
     n_items = 2 * (math.ceil(nsym / wl["segment"]) if wl["segment"] else 1)    # (chain, polarisation) pairs
-    aeq_cta = plan.aeq_kernel_for(n_items // 2, (wl["segment"] + wl["warmup"]) if wl["segment"] else nsym) == 2
-    if dom == "aeq":
-        kname = f"aeq_serial_kernel<{wl['n_aeq']}>" if aeq_cta else f"aeq_kernel<{wl['n_aeq']}>"
-        src = source_hash("aeq_serial.cu" if aeq_cta else "aeq.cu", "zf.cuh", "internal.h")
+    longest = (wl["segment"] + wl["warmup"]) if wl["segment"] else nsym
+    aeq_direct = args.aeq_kernel == 0 and wl.get("freq_sum", 0) != 1
+    aeq_split = aeq_direct and n_items < (3.2 if wl["n_aeq"] == 64 else 4.0) * 152
+    aeq_cta = not aeq_direct and plan.aeq_kernel_for(n_items // 2, longest) == 2
+    if dom == "aeq" and aeq_direct:
+        kname = f"aeq_{'split' if aeq_split else 'duo'}_kernel<{wl['n_aeq']}>"
+        src = source_hash("aeq_direct.cu", "internal.h")
+        ops, peak, basis = aeq_direct_ops(nsym), dot_peak_ops(2), "dp2a issue: 152 SMs x 64 lanes x 4 ops x 2070 MHz"
+    elif dom == "cdc" and args.cdc_kernel == 0:
+        kname, src = "cdc_direct_kernel<chain>", source_hash("cdc_direct.cu", "internal.h")
+        ops, peak = cdc_direct_ops(nsym, taps.shape[0]), dot_peak_ops(4)
+        basis = "dp4a issue: 152 SMs x 64 lanes x 8 ops x 2070 MHz"
     else:
-        kname, src = "cdc_kernel<chain>", source_hash("cdc.cu", "zf.cuh", "internal.h")
+        if dom == "aeq":
+            kname = f"aeq_serial_kernel<{wl['n_aeq']}>" if aeq_cta else f"aeq_kernel<{wl['n_aeq']}>"
+            src = source_hash("aeq_serial.cu" if aeq_cta else "aeq.cu", "zf.cuh", "internal.h")
+        else:
+            kname, src = "cdc_kernel<chain>", source_hash("cdc.cu", "zf.cuh", "internal.h")
+        ops = aeq_ops(nsym, wl["n_aeq"]) if dom == "aeq" else cdc_ops(n, S)
+        peak, basis = alu_peak_ops(), "152 SMs x 4 schedulers x 32 lanes x 2070 MHz (issue-bound int32), derived"
     achieved = ops / (dur * 1e-3) / 1e12
-    peak = alu_peak_ops() / 1e12
+    peak /= 1e12
     roof = {"bound": "alu", "kernel": kname, "achieved": round(achieved, 4), "peak": round(peak, 2),
-            "unit": "Tops/s (int32, algorithmic)", "frac": round(achieved / peak, 5),
-            "traffic": profiled_traffic(kname, src), "avg_launch_ms": round(dur, 4),
-            "peak_basis": "152 SMs x 4 schedulers x 32 lanes x 2070 MHz (issue-bound int32), derived"}
+            "unit": "Tops/s (int, algorithmic)", "frac": round(achieved / peak, 5),
+            "traffic": profiled_traffic(kname, src), "avg_launch_ms": round(dur, 4), "peak_basis": basis}
     prof = profiled_counters(kname, src)
     if prof:
         roof["ncu"] = prof
-    if dom == "aeq" and aeq_cta:
+    if dom == "aeq" and (aeq_cta or aeq_split):
         # a (chain, polarisation) is one serial recurrence and one CTA: the
         # launch can occupy at most n_items SMs
-        occ_peak = min(n_items, 152) * 4 * 32 * 2070e6 / 1e12
+        occ_peak = min(n_items, 152) / 152 * peak
         roof["occupied"] = {"sms": min(n_items, 152), "peak": round(occ_peak, 3),
                             "frac": round(achieved / occ_peak, 4),
                             "note": "the eq. (6) recurrence of each polarisation is serial over the stream's "
@@ -543,9 +572,11 @@ def run_fnt(args, rank, world, local_rank, oracle_pool=None):
                    "aeq_segment": wl["segment"],
                    "aeq_warmup": wl["warmup"], "aeq_update_period": wl.get("period", 1),
                    "aeq_freq_sum": wl.get("freq_sum", 0),
-                   "aeq_kernel": "a CTA per (chain, polarisation)" if aeq_cta else "a warp per (chain, polarisation)",
+                   "aeq_kernel": (f"direct, {'a CTA' if aeq_split else 'a warp'}" if aeq_direct else
+                                  "transforms, a CTA" if aeq_cta else "transforms, a warp") +
+                                 " per (chain, polarisation)",
                    "aeq_gradient": "tensor cores (exact f16 limbs, opt-in)" if args.tensor_gradient and not aeq_cta
-                   else "integer pipes",
+                   and not aeq_direct else "integer pipes",
                    "samples_per_step": n, "symbols_per_step": nsym,
                    "l2": f"inputs rotate over {ring} device buffers of {x_np.nbytes >> 20} MiB "
                          f"({ring * x_np.nbytes >> 20} MiB" + (" > 2x the 129 MB L2), no flush"
@@ -704,22 +735,28 @@ def run_cfg1(args):
     torch.cuda.synchronize()
     per = sorted(e[0].elapsed_time(e[1]) for e in evs)
     ms = statistics.mean(per)
-    ops = cdc_ops(n, 48, n_pol=1)
     n_items = math.ceil(math.ceil(n / 48) / 32)
-    split = plan.cdc_kernel_for(n_items) == 2
-    kname = "cdc_split_kernel<cdc>" if split else "cdc_kernel<cdc>"
-    src = source_hash("cdc.cu", "zf.cuh", "internal.h")
+    if args.cdc_kernel == 0:
+        kname, src = "cdc_direct_kernel<cdc>", source_hash("cdc_direct.cu", "internal.h")
+        ops, peak = cdc_direct_ops(n, 17, n_pol=1), dot_peak_ops(4)
+        note = "65,536 samples are 256 tiles of 256, a warp each"
+    else:
+        split = plan.cdc_kernel_for(n_items) == 2
+        kname = "cdc_split_kernel<cdc>" if split else "cdc_kernel<cdc>"
+        src = source_hash("cdc.cu", "zf.cuh", "internal.h")
+        ops, peak = cdc_ops(n, 48, n_pol=1), alu_peak_ops()
+        note = "65,536 samples is 1366 blocks in 43 work items of 32 blocks: " + (
+            "a block per 8 threads, 344 warps" if split else "a block per lane, 43 warps")
     return {"workload": "cfg1: single-pol FNT-CDC, 65,536 samples, 17 taps, N=64 alpha=4080 S=48",
             "metric": "Msamples/s", "value": round(n / (ms * 1e-3) / 1e6, 2), "ms_per_step": round(ms, 4),
             "steps": args.steps, "gpu_launches_per_step": b.kernel_count(),
             "repeat": {"launches": len(per), "best_ms": round(per[0], 4), "median_ms": round(statistics.median(per), 4)},
             "roofline": {"bound": "alu", "kernel": kname, "achieved": round(ops / (ms * 1e-3) / 1e12, 3),
-                         "peak": round(alu_peak_ops() / 1e12, 2), "unit": "Tops/s (int32, algorithmic)",
-                         "frac": round(ops / (ms * 1e-3) / alu_peak_ops(), 4),
+                         "peak": round(peak / 1e12, 2), "unit": "Tops/s (int, algorithmic)",
+                         "frac": round(ops / (ms * 1e-3) / peak, 4),
                          "traffic": profiled_traffic(kname, src), "ncu": profiled_counters(kname, src),
                          "timing": "graph launch included"},
-            "note": "65,536 samples is 1366 blocks in 43 work items of 32 blocks: " +
-                    ("a block per 8 threads, 344 warps" if split else "a block per lane, 43 warps")}
+            "note": note}
 
 
 def run_cfg3(args):
@@ -886,7 +923,7 @@ def run_cfg4(args):
         res[name] = {"paced": paced, "saturated": flood, "oracle_links_bitexact": ok, "oracle_frames_checked": nchk,
                      "aeq": "one serial run per frame (eq. (6) over the frame)" if not over else
                             f"segments of {over['aeq_segment']} + {over['aeq_warmup']} from the link's taps",
-                     "aeq_kernel": {0: "automatic (a CTA per chain when a wave's chains fit one per SM)",
+                     "aeq_kernel": {0: "direct form (automatic)",
                                     1: "a warp per chain (forced)", 2: "a CTA per chain (forced)"}[kernel]}
     offered_gsps = sum(f.x.shape[0] for f in tr.frames) / tr.frames[-1].arrival_s / 1e9
     return {"workload": f"cfg4: {len(tr.frames)} frames, Poisson 20k frames/s over {len(tr.link_taps)} links, "
