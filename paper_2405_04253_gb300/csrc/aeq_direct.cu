@@ -43,12 +43,12 @@ namespace fnt {
 
 namespace {
 
-template <int NA>
+template <int NA, int PB_>
 struct DirCfg {
     static constexpr int K = kAeqK;
     static constexpr int SA = NA - K;                     // symbols per block
     static constexpr int NG = SA / 4;                     // groups of four symbols
-    static constexpr int PB = NA == 64 ? 4 : 8;           // blocks per staged batch
+    static constexpr int PB = PB_;                        // blocks per staged batch
     static constexpr int B = PB * SA;                     // symbols per staged batch
     static constexpr int XW = K + B;                      // staged words: K of history
     static_assert(K == 16 && SA % 16 == 0, "shapes");
@@ -129,8 +129,8 @@ __device__ __forceinline__ void stage(uint32_t *xn, const uint32_t *xin, int64_t
 
 // xq[q] <- the byte transpose of the staged words q .. q + 3, by NTHR threads, four
 // words of q a thread at a time (loads before stores).
-template <class C, int NTHR = 32>
-__device__ __forceinline__ void transpose(const uint32_t *xn, uint4 *xq, int lane) {
+template <class C, int NTHR = 32, bool PLANES = false>
+__device__ __forceinline__ void transpose(const uint32_t *xn, uint4 *xq, int lane, uint32_t *xp = nullptr) {
     constexpr int NQ = C::XW - 3;
 #pragma unroll
     for (int q0 = 0; q0 < NQ; q0 += 4 * NTHR) {
@@ -144,9 +144,15 @@ __device__ __forceinline__ void transpose(const uint32_t *xn, uint4 *xq, int lan
             const int q = q0 + NTHR * j + lane;
             const uint32_t ab0 = __byte_perm(w[j][0], w[j][1], 0x5140), ab1 = __byte_perm(w[j][0], w[j][1], 0x7362);
             const uint32_t cd0 = __byte_perm(w[j][2], w[j][3], 0x5140), cd1 = __byte_perm(w[j][2], w[j][3], 0x7362);
-            if (q0 + NTHR * j < NQ && q < NQ)
-                xq[q] = make_uint4(__byte_perm(ab0, cd0, 0x5410), __byte_perm(ab0, cd0, 0x7632),
-                                   __byte_perm(ab1, cd1, 0x5410), __byte_perm(ab1, cd1, 0x7632));
+            if (q0 + NTHR * j < NQ && q < NQ) {
+                const uint4 v = make_uint4(__byte_perm(ab0, cd0, 0x5410), __byte_perm(ab0, cd0, 0x7632),
+                                           __byte_perm(ab1, cd1, 0x5410), __byte_perm(ab1, cd1, 0x7632));
+                xq[q] = v;
+                if constexpr (PLANES) {
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) xp[s * C::XW + q] = word_of(v, s);
+                }
+            }
         }
     }
 }
@@ -221,12 +227,15 @@ __device__ __forceinline__ int32_t out_of(int32_t y) { return min(max(y >> 7, -3
 // Limbs go from output to gradient warps at barrier 1, which also tells whether any
 // e z needs its third limb, taps back at barrier 3 (the writers arrive, the readers
 // wait); barrier 2 joins all warps once a batch.
-// What a block takes is the latency of that round trip: 0.24 us at N = 32 and 0.35 us
+// What a block takes is the latency of that round trip: 0.23 us at N = 32 and 0.31 us
 // at N = 64 for a lone chain (0.60 and 0.83 us with the transforms on a CTA); with a
 // whole block in one warp it was 0.34 and 0.61 us, about 200 and 500 dependent
 // instructions at 3 to 4 cycles each.
 template <int NA>
 struct SplitCfg {
+    // batches of 16 (N = 32) and 8 blocks: half that costs 2.5 % of a block, twice
+    // that more again (0.228, 0.325 us against 0.234, 0.333 and 0.251, 0.338)
+    using C = DirCfg<NA, NA == 64 ? 8 : 16>;
     static constexpr int NC = (NA - kAeqK) / 16;          // output warps
     static constexpr int NGW = 4;                         // gradient warps
     static constexpr int NCG = 32 * (NC + NGW);
@@ -255,11 +264,12 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
                                                                      const AeqChain *__restrict__ chains,
                                                                      AeqParams prm,
                                                                      const __grid_constant__ SingleFrame one) {
-    using C = DirCfg<NA>;
     using R = SplitCfg<NA>;
+    using C = typename R::C;
     constexpr int K = C::K, SA = C::SA, NG = C::NG, NC = R::NC, NCG = R::NCG;
     constexpr int WO = 12;                        // 16-byte words per tap row: the outputs 16 banks apart
     __shared__ uint4 s_xq[2][C::XW];
+    __shared__ uint32_t s_xp[2][4 * C::XW];       // the same words, an input after the other
     __shared__ uint32_t s_xn[C::XW];
     __shared__ uint4 s_w[2 * WO];
     __shared__ uint4 s_ez[2 * NG];
@@ -285,7 +295,7 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
         for (int64_t j = 0; j < nbatch; ++j) {
             cp_async_wait_all();
             __syncwarp();
-            transpose<C>(s_xn, s_xq[j & 1], lane);
+            transpose<C, 32, true>(s_xn, s_xq[j & 1], lane, s_xp[j & 1]);
             __syncwarp();
             if (j + 1 < nbatch) stage<C>(s_xn, xin, ch.begin + (j + 1) * C::B, ch.lo, ch.end, lane);
             bar_sync<2, R::NT>();                 // batch j staged; batch j - 1 consumed
@@ -349,11 +359,11 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
             bar_sync<2, R::NT>();
             if (mu >= 63) continue;                // the taps never move
             const int nb = (int)min((int64_t)C::PB, nblk - j * C::PB);
-            const uint32_t *xs = (const uint32_t *)(s_xq[j & 1] + K - i) + s1;
-            for (int bb = 0; bb < nb; ++bb, xs += 4 * SA) {
+            const uint32_t *xs = s_xp[j & 1] + s1 * C::XW + K - i;
+            for (int bb = 0; bb < nb; ++bb, xs += SA) {
                 uint32_t x[NG];
 #pragma unroll
-                for (int n = 0; n < NG; ++n) x[n] = xs[16 * n];
+                for (int n = 0; n < NG; ++n) x[n] = xs[4 * n];
                 const bool any = bar_or<1, NCG>(false);   // limbs stored; some c2 is not 0
                 int32_t l0[4] = {0, 0, 0, 0}, l1[4] = {0, 0, 0, 0};
 #pragma unroll
@@ -402,14 +412,16 @@ __global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFr
 // reduced over lanes and two __syncwarp order a block.  The warps share the staged
 // batch and meet twice a batch.  Lanes 2 i and 2 i + 1 read the same staged word, so a
 // 16-byte load of the warp is two passes over shared memory, not four.  Bound by issue
-// once four warps share a scheduler: 0.73 us a block for 1,216 chains at N = 32, 1.64
+// once four warps share a scheduler: 0.69 us a block for 1,216 chains at N = 32, 1.62
 // us at N = 64.  (One warp for both polarisations shares more loads, but took 0.73 and
-// 1.65 us there and 0.49 to 0.73 us where this one takes 0.45 to 0.58.)
+// 1.65 us there, and 0.49 and 0.73 us for 608 and 760 chains at N = 32 where this one
+// takes 0.43 and 0.55.)
 template <int NA, bool PER>
 __global__ void __launch_bounds__(64) aeq_duo_kernel(const DevFrame *__restrict__ frames,
                                                      const AeqChain *__restrict__ chains, AeqParams prm,
                                                      const __grid_constant__ SingleFrame one) {
-    using C = DirCfg<NA>;
+    // batches of 32 (N = 32) and 8 blocks: with 8 and 4, 1 to 10 % slower
+    using C = DirCfg<NA, NA == 64 ? 8 : 32>;
     constexpr int K = C::K, SA = C::SA, NG = C::NG, M = SA / 16;
     constexpr int WO = 12;
     __shared__ uint4 s_xq[C::XW];
@@ -576,8 +588,8 @@ const SingleFrame kNoSingle{};
 // one's length the launch amounts to.  Measured with equal chains, us a block (split,
 // duo), by (chain, polarisation) items per SM (152 SMs):
 //            1            2            3            4            5            6
-//   N = 64   .352  .621   .466  .628   .601  .628   .749  .634   1.00  .914   1.13  .913
-//   N = 32   .243  .339   .260  .340   .317  .345   .354  .346   .429  .444   .622  .444
+//   N = 64   .314  .590   .412  .588   .535  .595   .794  .601   .914  .895   1.05  .891
+//   N = 32   .230  .322   .246  .324   .296  .327   .332  .330   .406  .419   .588  .419
 cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
                               int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
                               cudaStream_t stream, const SingleFrame *one) {
