@@ -230,7 +230,9 @@ __device__ __forceinline__ int32_t out_of(int32_t y) { return min(max(y >> 7, -3
 // What a block takes is the latency of that round trip: 0.23 us at N = 32 and 0.31 us
 // at N = 64 for a lone chain (0.60 and 0.83 us with the transforms on a CTA); with a
 // whole block in one warp it was 0.34 and 0.61 us, about 200 and 500 dependent
-// instructions at 3 to 4 cycles each.
+// instructions at 3 to 4 cycles each.  The launch bound of four CTAs an SM (64
+// registers at N = 64) lets four items share an SM and takes 8 to 10 % off a block
+// against no bound; a bound of two or three gives less, five and six cost time.
 template <int NA>
 struct SplitCfg {
     // batches of 16 (N = 32) and 8 blocks: half that costs 2.5 % of a block, twice
@@ -260,7 +262,7 @@ __device__ __forceinline__ bool bar_or(bool v) {
 }
 
 template <int NA, bool PER>
-__global__ void __launch_bounds__(SplitCfg<NA>::NT) aeq_split_kernel(const DevFrame *__restrict__ frames,
+__global__ void __launch_bounds__(SplitCfg<NA>::NT, 4) aeq_split_kernel(const DevFrame *__restrict__ frames,
                                                                      const AeqChain *__restrict__ chains,
                                                                      AeqParams prm,
                                                                      const __grid_constant__ SingleFrame one) {
