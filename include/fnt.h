@@ -295,8 +295,9 @@ FNT_API int32_t fnt_batch_kernel_count(const fnt_batch *b);
 
 FNT_API fnt_status fnt_batch_destroy(fnt_batch *b);
 
-/* Sets the warps per CTA of the CDC and AEQ kernels used by later launches of
- * this plan (autotuner hook).  0 keeps the current value. */
+/* Sets the warps per CTA of the transform CDC and AEQ kernels in later launches of
+ * this plan (autotuner hook; the direct forms have their own).  0 keeps the current
+ * value. */
 FNT_API fnt_status fnt_plan_set_launch(fnt_plan *plan, int32_t cdc_warps, int32_t aeq_warps);
 
 /* Prepared chain batches created after this call split their work into

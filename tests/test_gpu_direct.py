@@ -136,3 +136,27 @@ def test_aeq_state_beyond_range(orc, na, alpha, copies):
     torch.cuda.synchronize()
     ref, Tr = orc.aeq(x, T0, na, alpha, mu_shift=9, rde_a=64)
     assert (out.cpu().numpy() == ref).all() and (st.cpu().numpy() == Tr).all()
+
+
+@pytest.mark.parametrize("pin", [True, False])
+@pytest.mark.parametrize("op", ["cdc", "aeq"])
+def test_host_buffers(orc, op, pin):
+    """One-shot calls on host buffers of one frame: page-locked ones in place,
+    pageable ones staged."""
+    rng = np.random.default_rng(17)
+    n = 5001
+    x = rng.integers(-16, 16, (n, 2, 2)).astype(np.int8)
+    taps = rng.integers(-32, 32, (17, 2)).astype(np.int8)
+    xt, out = torch.from_numpy(x), torch.full((n, 2, 2) if op == "cdc" else (n, 4), 0x3C3C, dtype=torch.int16)
+    if pin:
+        xt, out = xt.pin_memory(), out.pin_memory()
+    plan = F.Plan(mu_shift=9, aeq_segment=700, aeq_warmup=33)
+    if op == "cdc":
+        F.cdc_run(plan, [F.Frame(xt, out, taps)], host=True)
+        assert np.array_equal(out.numpy().astype(np.int32), orc.cdc(x, taps))
+        return
+    T0 = orc.aeq_init_taps(16, 2048)
+    st = dev(T0)
+    F.aeq_run(plan, [F.Frame(xt.reshape(n, 4), out, state=st)], host=True)
+    ref, Tr = orc.aeq_segmented(x.reshape(n, 4), T0, 32, 2, 9, 64, 700, 33, True, 1, 0)
+    assert np.array_equal(out.numpy(), ref) and np.array_equal(st.cpu().numpy(), Tr)
