@@ -524,7 +524,7 @@ def run_fnt(args, rank, world, local_rank, oracle_pool=None):
     n_items = 2 * (math.ceil(nsym / wl["segment"]) if wl["segment"] else 1)    # (chain, polarisation) pairs
     longest = (wl["segment"] + wl["warmup"]) if wl["segment"] else nsym
     aeq_direct = args.aeq_kernel == 0 and wl.get("freq_sum", 0) != 1
-    aeq_split = aeq_direct and n_items < (3.2 if wl["n_aeq"] == 64 else 4.0) * 152
+    aeq_split = aeq_direct and n_items < (3.5 if wl["n_aeq"] == 64 else 2.8 if wl.get("period", 1) > 1 else 4.0) * 152
     aeq_cta = not aeq_direct and plan.aeq_kernel_for(n_items // 2, longest) == 2
     if dom == "aeq" and aeq_direct:
         kname = f"aeq_{'split' if aeq_split else 'duo'}_kernel<{wl['n_aeq']}>"

@@ -227,7 +227,7 @@ __device__ __forceinline__ int32_t out_of(int32_t y) { return min(max(y >> 7, -3
 // Limbs go from output to gradient warps at barrier 1, which also tells whether any
 // e z needs its third limb, taps back at barrier 3 (the writers arrive, the readers
 // wait); barrier 2 joins all warps once a batch.
-// What a block takes is the latency of that round trip: 0.23 us at N = 32 and 0.31 us
+// What a block takes is the latency of that round trip: 0.21 us at N = 32 and 0.29 us
 // at N = 64 for a lone chain (0.60 and 0.83 us with the transforms on a CTA); with a
 // whole block in one warp it was 0.34 and 0.61 us, about 200 and 500 dependent
 // instructions at 3 to 4 cycles each.  The launch bound of four CTAs an SM (64
@@ -236,7 +236,8 @@ __device__ __forceinline__ int32_t out_of(int32_t y) { return min(max(y >> 7, -3
 template <int NA>
 struct SplitCfg {
     // batches of 16 (N = 32) and 8 blocks: half that costs 2.5 % of a block, twice
-    // that more again (0.228, 0.325 us against 0.234, 0.333 and 0.251, 0.338)
+    // that more again (0.228, 0.325 us against 0.234, 0.333 and 0.251, 0.338, before
+    // the launch bound)
     using C = DirCfg<NA, NA == 64 ? 8 : 16>;
     static constexpr int NC = (NA - kAeqK) / 16;          // output warps
     static constexpr int NGW = 4;                         // gradient warps
@@ -589,9 +590,13 @@ const SingleFrame kNoSingle{};
 // fewer cycles of an SM a block.  total / longest is how many chains of the longest
 // one's length the launch amounts to.  Measured with equal chains, us a block (split,
 // duo), by (chain, polarisation) items per SM (152 SMs):
-//            1            2            3            4            5            6
-//   N = 64   .314  .590   .412  .588   .535  .595   .794  .601   .914  .895   1.05  .891
-//   N = 32   .230  .322   .246  .324   .296  .327   .332  .330   .406  .419   .588  .419
+//                  1            2            3            4            5            6
+//   N = 64         .293  .590   .397  .590   .518  .597   .649  .601   .861  .892   .984  .894
+//   N = 32         .209  .322   .227  .322   .288  .326   .322  .327   .489  .419   .518  .419
+//   N = 64, P = 4  .309  .559   .414  .562   .545  .569   .685  .568   .886  .877   1.02  .876
+//   N = 32, P = 4  .212  .292   .238  .291   .307  .295   .350  .297   .505  .393   .544  .392
+// so the lines lie between 3 and 4 items, at 4, and (update period P > 1, N = 32)
+// between 2 and 3.
 cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
                               int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
                               cudaStream_t stream, const SingleFrame *one) {
@@ -599,7 +604,7 @@ cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *ch
     const SingleFrame &single = one ? *one : kNoSingle;
     if (one) frames = nullptr, chains = nullptr;
     const double items = 2.0 * (double)total_symbols / (double)std::max<int64_t>(longest_symbols, 1);
-    const bool split = items < (na == 64 ? 3.2 : 4.0) * n_sm;
+    const bool split = items < (na == 64 ? 3.5 : prm.period > 1 ? 2.8 : 4.0) * n_sm;
     if (na == 64)
         launch_na<64>(split, frames, chains, n_chains, prm, stream, single);
     else

@@ -46,7 +46,7 @@ template <bool CHAIN, int NPOL>
 struct CdcDirect {
     static constexpr int ROW = CHAIN ? kHistPairs + kTile : kHistPairs + kHalf + (NPOL == 2 ? 8 : 0);
     static constexpr int WORDS = CHAIN ? NPOL * ROW : 2 * NPOL * ROW;
-    static_assert(ROW % 4 == 0, "16-byte rows");
+    static_assert(ROW % 4 == 0 && WORDS % 4 == 0, "16-byte rows");
     // row start of group g (CDC: parity, chain: half) and polarisation p
     static __device__ __forceinline__ int base(int g, int p) {
         return CHAIN ? p * ROW + g * kHalf : (g * NPOL + p) * ROW;
