@@ -522,21 +522,22 @@ def run_fnt(args, rank, world, local_rank, oracle_pool=None):
     dom = "aeq" if aeq_avg >= cdc_avg else "cdc"
     dur = aeq_avg if dom == "aeq" else cdc_avg
     n_items = 2 * (math.ceil(nsym / wl["segment"]) if wl["segment"] else 1)    # (chain, polarisation) pairs
-    longest = (wl["segment"] + wl["warmup"]) if wl["segment"] else nsym
-    aeq_direct = args.aeq_kernel == 0 and wl.get("freq_sum", 0) != 1
-    aeq_split = aeq_direct and n_items < (3.5 if wl["n_aeq"] == 64 else 2.8 if wl.get("period", 1) > 1 else 4.0) * 152
-    aeq_cta = not aeq_direct and plan.aeq_kernel_for(n_items // 2, longest) == 2
+    longest = min(nsym, wl["segment"] + wl["warmup"]) if wl["segment"] else nsym
+    aeq_total = nsym + sum(min(k, wl["warmup"]) for k in range(0, nsym, wl["segment"])) if wl["segment"] else nsym
+    aeq_name = plan.aeq_route(n_items // 2, aeq_total, longest)
+    aeq_direct = aeq_name in ("aeq_split_kernel", "aeq_duo_kernel")
+    aeq_split, aeq_cta = aeq_name == "aeq_split_kernel", aeq_name == "aeq_serial_kernel"
     if dom == "aeq" and aeq_direct:
-        kname = f"aeq_{'split' if aeq_split else 'duo'}_kernel<{wl['n_aeq']}>"
+        kname = f"{aeq_name}<{wl['n_aeq']}>"
         src = source_hash("aeq_direct.cu", "internal.h")
         ops, peak, basis = aeq_direct_ops(nsym), dot_peak_ops(2), "dp2a issue: 152 SMs x 64 lanes x 4 ops x 2070 MHz"
-    elif dom == "cdc" and args.cdc_kernel == 0:
+    elif dom == "cdc" and plan.cdc_route() == "cdc_direct_kernel":
         kname, src = "cdc_direct_kernel<chain>", source_hash("cdc_direct.cu", "internal.h")
         ops, peak = cdc_direct_ops(nsym, taps.shape[0]), dot_peak_ops(4)
         basis = "dp4a issue: 152 SMs x 64 lanes x 8 ops x 2070 MHz"
     else:
         if dom == "aeq":
-            kname = f"aeq_serial_kernel<{wl['n_aeq']}>" if aeq_cta else f"aeq_kernel<{wl['n_aeq']}>"
+            kname = f"{aeq_name}<{wl['n_aeq']}>"
             src = source_hash("aeq_serial.cu" if aeq_cta else "aeq.cu", "zf.cuh", "internal.h")
         else:
             kname, src = "cdc_kernel<chain>", source_hash("cdc.cu", "zf.cuh", "internal.h")
@@ -718,6 +719,7 @@ def run_cfg1(args):
     f = synth.config1()
     n = f.x.shape[0]
     plan = fnt.Plan()
+    plan.set_cdc_kernel(args.cdc_kernel)
     x = torch.from_numpy(f.x).cuda()
     out = torch.zeros((n, 1, 2), dtype=torch.int16, device="cuda")
     b = fnt.Batch(plan, [fnt.Frame(x, out, f.taps, n_pol=1)], fnt.OP_CDC, use_graph=True)
@@ -736,17 +738,17 @@ def run_cfg1(args):
     per = sorted(e[0].elapsed_time(e[1]) for e in evs)
     ms = statistics.mean(per)
     n_items = math.ceil(math.ceil(n / 48) / 32)
-    if args.cdc_kernel == 0:
-        kname, src = "cdc_direct_kernel<cdc>", source_hash("cdc_direct.cu", "internal.h")
+    route = plan.cdc_route(n_items)
+    kname = route + "<cdc>"
+    if route == "cdc_direct_kernel":
+        src = source_hash("cdc_direct.cu", "internal.h")
         ops, peak = cdc_direct_ops(n, 17, n_pol=1), dot_peak_ops(4)
         note = "65,536 samples are 256 tiles of 256, a warp each"
     else:
-        split = plan.cdc_kernel_for(n_items) == 2
-        kname = "cdc_split_kernel<cdc>" if split else "cdc_kernel<cdc>"
         src = source_hash("cdc.cu", "zf.cuh", "internal.h")
         ops, peak = cdc_ops(n, 48, n_pol=1), alu_peak_ops()
         note = "65,536 samples is 1366 blocks in 43 work items of 32 blocks: " + (
-            "a block per 8 threads, 344 warps" if split else "a block per lane, 43 warps")
+            "a block per 8 threads, 344 warps" if route == "cdc_split_kernel" else "a block per lane, 43 warps")
     return {"workload": "cfg1: single-pol FNT-CDC, 65,536 samples, 17 taps, N=64 alpha=4080 S=48",
             "metric": "Msamples/s", "value": round(n / (ms * 1e-3) / 1e6, 2), "ms_per_step": round(ms, 4),
             "steps": args.steps, "gpu_launches_per_step": b.kernel_count(),
@@ -1033,9 +1035,11 @@ def main(argv=None):
     ap.add_argument("--ref-segments", type=int, default=48)
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--cdc-kernel", type=int, default=0, choices=(0, 1, 2),
-                    help="cfg2 / cfg5: CDC kernel (0 automatic, 1 a block per lane, 2 a block per 8 threads)")
+                    help="cfg1 / cfg2 / cfg5: CDC kernel (0 direct form, 1 transforms, a block per lane, "
+                         "2 transforms, a block per 8 threads)")
     ap.add_argument("--aeq-kernel", type=int, default=0, choices=(0, 1, 2),
-                    help="cfg2 / cfg5: AEQ kernel (0 automatic, 1 a warp, 2 a CTA per chain and polarisation)")
+                    help="cfg2 / cfg5: AEQ kernel (0 direct form, 1 transforms, a warp, 2 transforms, a CTA per chain "
+                         "and polarisation)")
     ap.add_argument("--tensor-gradient", action="store_true",
                     help="cfg2 / cfg5: AEQ gradient on the tensor cores (bit-identical; off = integer path)")
     ap.add_argument("--aeq-freq-sum", type=int, default=0, choices=(0, 1, 2),

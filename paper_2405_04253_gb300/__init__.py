@@ -119,6 +119,14 @@ SIGNATURES = {
     "fnt_session_destroy": (_I32, [_VP]),
 }
 
+# Exported for the benchmark and the tests, not part of include/fnt.h.
+INTERNAL_SIGNATURES = {
+    "fnt_internal_cdc_route": (_I32, [_VP, _I64]),
+    "fnt_internal_aeq_route": (_I32, [_VP, _I64, _I64, _I64]),
+}
+CDC_ROUTES = (None, "cdc_kernel", "cdc_split_kernel", "cdc_direct_kernel")
+AEQ_ROUTES = (None, "aeq_kernel", "aeq_serial_kernel", "aeq_split_kernel", "aeq_duo_kernel")
+
 _lib = None
 
 
@@ -128,7 +136,7 @@ def lib(path: str | None = None):
     if _lib is None:
         p = path or os.environ.get("FNT_LIB") or build()
         L = ctypes.CDLL(p)
-        for name, (res, args) in SIGNATURES.items():
+        for name, (res, args) in (SIGNATURES | INTERNAL_SIGNATURES).items():
             fn = getattr(L, name)
             fn.restype = res
             fn.argtypes = args
@@ -243,6 +251,17 @@ class Plan:
         """The transform AEQ kernel (1 or 2) for a launch of n_chains chains, the
         longest of longest_symbols symbols."""
         return int(lib().fnt_plan_aeq_kernel_for(self.handle, int(n_chains), int(longest_symbols)))
+
+    def cdc_route(self, n_items: int = 1) -> str:
+        """The CDC kernel of calls and batches made now with this plan (transform
+        kernels: for n_items 32-block work items)."""
+        return CDC_ROUTES[lib().fnt_internal_cdc_route(self.handle, int(n_items))]
+
+    def aeq_route(self, n_chains: int, total_symbols: int, longest_symbols: int) -> str:
+        """The AEQ kernel a launch of n_chains chains takes, of total_symbols in all
+        (warm-ups included), the longest of longest_symbols."""
+        return AEQ_ROUTES[lib().fnt_internal_aeq_route(self.handle, int(n_chains), int(total_symbols),
+                                                       int(longest_symbols))]
 
     def initial_state(self) -> np.ndarray:
         """The plan's initial AEQ taps, int32 [4 (S2)][4 (S1)][16]."""

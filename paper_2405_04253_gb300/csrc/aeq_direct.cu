@@ -27,7 +27,7 @@
 // symbols of an input) read aligned 16-byte words at any offset.  A batch of
 // blocks is transposed at once while the next batch's words arrive by cp.async.
 //
-// Two layouts; aeq_direct_launch picks one (rule and figures there).
+// Two layouts; aeq_direct_split picks one (rule and figures there).
 //   aeq_duo_kernel    a warp per (chain, polarisation): many chains, bound by dp2a issue
 //                     and shared-memory loads
 //   aeq_split_kernel  six or eight warps per (chain, polarisation), by role: few
@@ -597,14 +597,16 @@ const SingleFrame kNoSingle{};
 //   N = 32, P = 4  .212  .292   .238  .291   .307  .295   .350  .297   .505  .393   .544  .392
 // so the lines lie between 3 and 4 items, at 4, and (update period P > 1, N = 32)
 // between 2 and 3.
-cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
-                              int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
-                              cudaStream_t stream, const SingleFrame *one) {
+bool aeq_direct_split(int na, int period, int64_t total_symbols, int64_t longest_symbols, int n_sm) {
+    const double items = 2.0 * (double)total_symbols / (double)std::max<int64_t>(longest_symbols, 1);
+    return items < (na == 64 ? 3.5 : period > 1 ? 2.8 : 4.0) * n_sm;
+}
+
+cudaError_t aeq_direct_launch(int na, bool split, const DevFrame *frames, const AeqChain *chains, int n_chains,
+                              AeqParams prm, cudaStream_t stream, const SingleFrame *one) {
     if (n_chains <= 0) return cudaSuccess;
     const SingleFrame &single = one ? *one : kNoSingle;
     if (one) frames = nullptr, chains = nullptr;
-    const double items = 2.0 * (double)total_symbols / (double)std::max<int64_t>(longest_symbols, 1);
-    const bool split = items < (na == 64 ? 3.5 : prm.period > 1 ? 2.8 : 4.0) * n_sm;
     if (na == 64)
         launch_na<64>(split, frames, chains, n_chains, prm, stream, single);
     else

@@ -335,12 +335,32 @@ cudaError_t fnt::aeq_launch_for(const fnt_plan *p, const DevFrame *frames, const
                                 int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream,
                                 const SingleFrame *one) {
     AeqParams prm{p->d.mu_shift, p->d.rde_a, update_period(p->d), p->tensor_gradient, p->d.aeq_freq_sum};
-    if (aeq_use_direct(p))
-        return aeq_direct_launch(p->d.n_aeq, frames, chains, n_chains, total_symbols, longest_symbols, prm, p->n_sm,
-                                 stream, one);
-    if (aeq_use_serial(p, n_chains, longest_symbols))
+    const AeqRoute route = aeq_route(p, n_chains, total_symbols, longest_symbols);
+    switch (route) {
+    case kAeqCta:
         return aeq_serial_launch(p->d.n_aeq, frames, chains, n_chains, prm, 0, stream);
-    return aeq_launch(p->d.n_aeq, frames, chains, n_chains, prm, p->aeq_warps, 0, stream, aeq_min_smem(p));
+    case kAeqWarp:
+        return aeq_launch(p->d.n_aeq, frames, chains, n_chains, prm, p->aeq_warps, 0, stream, aeq_min_smem(p));
+    default:
+        return aeq_direct_launch(p->d.n_aeq, route == kAeqSplit, frames, chains, n_chains, prm, stream, one);
+    }
+}
+
+AeqRoute fnt::aeq_route(const fnt_plan *p, int64_t n_chains, int64_t total_symbols, int64_t longest_symbols) {
+    if (aeq_use_direct(p))
+        return aeq_direct_split(p->d.n_aeq, update_period(p->d), total_symbols, longest_symbols, p->n_sm) ? kAeqSplit
+                                                                                                       : kAeqDuo;
+    return aeq_use_serial(p, n_chains, longest_symbols) ? kAeqCta : kAeqWarp;
+}
+
+extern "C" int32_t fnt_internal_aeq_route(const fnt_plan *p, int64_t n_chains, int64_t total_symbols,
+                                          int64_t longest_symbols) {
+    return p ? aeq_route(p, n_chains, total_symbols, longest_symbols) : 0;
+}
+
+extern "C" int32_t fnt_internal_cdc_route(const fnt_plan *p, int64_t n_items) {
+    if (!p) return 0;
+    return cdc_use_direct(p) ? kCdcDirect : cdc_use_split(p, n_items) ? kCdcSplit : kCdcLane;
 }
 
 extern "C" fnt_status fnt_plan_initial_taps(const fnt_plan *p, int32_t *state) {

@@ -126,10 +126,17 @@ bool aeq_use_serial(const fnt_plan *p, int64_t n_chains, int64_t longest_symbols
 cudaError_t aeq_launch_for(const fnt_plan *p, const DevFrame *frames, const AeqChain *chains, int n_chains,
                            int64_t total_symbols, int64_t longest_symbols, cudaStream_t stream,
                            const SingleFrame *one = nullptr);
-// The direct form of the AEQ (aeq_direct.cu).
-cudaError_t aeq_direct_launch(int na, const DevFrame *frames, const AeqChain *chains, int n_chains,
-                              int64_t total_symbols, int64_t longest_symbols, AeqParams prm, int n_sm,
-                              cudaStream_t stream, const SingleFrame *one = nullptr);
+// The direct form of the AEQ (aeq_direct.cu), in its split or duo layout, and which of
+// them a launch takes.
+cudaError_t aeq_direct_launch(int na, bool split, const DevFrame *frames, const AeqChain *chains, int n_chains,
+                              AeqParams prm, cudaStream_t stream, const SingleFrame *one = nullptr);
+bool aeq_direct_split(int na, int period, int64_t total_symbols, int64_t longest_symbols, int n_sm);
+// The kernels of aeq.cu, aeq_serial.cu and aeq_direct.cu; the one a launch of n_chains
+// chains takes, of total_symbols in all, the longest of longest_symbols.
+enum AeqRoute { kAeqWarp = 1, kAeqCta = 2, kAeqSplit = 3, kAeqDuo = 4 };
+AeqRoute aeq_route(const fnt_plan *p, int64_t n_chains, int64_t total_symbols, int64_t longest_symbols);
+// The CDC kernels: a block per lane, a block per 8 threads, direct.
+enum CdcRoute { kCdcLane = 1, kCdcSplit = 2, kCdcDirect = 3 };
 // Whether the plan's CDC and AEQ run in direct form (no transform kernel picked).
 bool cdc_use_direct(const fnt_plan *p);
 bool aeq_use_direct(const fnt_plan *p);
@@ -145,3 +152,11 @@ int64_t single_chains(const SingleFrame &one);
 fnt_status launch_single(const fnt_plan *p, const SingleFrame &one, int op, cudaStream_t stream, int stages);
 
 }  // namespace fnt
+
+// What runs, for the benchmark and the tests (exported, not part of include/fnt.h):
+// the CdcRoute of calls and batches made now with the plan (n_items transform items),
+// and the AeqRoute of a launch; 0 for a null plan.
+extern "C" __attribute__((visibility("default"))) int32_t fnt_internal_cdc_route(const fnt_plan *p, int64_t n_items);
+extern "C" __attribute__((visibility("default"))) int32_t fnt_internal_aeq_route(const fnt_plan *p, int64_t n_chains,
+                                                                                int64_t total_symbols,
+                                                                                int64_t longest_symbols);

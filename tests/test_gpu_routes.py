@@ -1,0 +1,83 @@
+"""Which kernel a call, a prepared batch or a session runs, by the names the CUDA
+profiler records: the launch rules, the plan settings that pick a kernel, and the
+same rule for a frame passed as a parameter and through work tables."""
+import re
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2405_04253_gb300 as F  # noqa: E402
+
+
+def kernels(fn):
+    """Names of the library's kernels that fn launches, in order of their start."""
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(3):                       # the first session of a process may record nothing
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            fn()
+            torch.cuda.synchronize()
+        ev = sorted((e for e in prof.events() if "fnt::" in e.name), key=lambda e: e.time_range.start)
+        if ev:
+            return [re.search(r"::(\w+)[<(]", e.name.replace("(anonymous namespace)::", "")).group(1) for e in ev]
+    pytest.skip("the CUDA profiler records no kernels here")
+
+
+def symbols(rng, n):
+    return torch.from_numpy(rng.integers(-16, 16, (n, 4)).astype(np.int8)).cuda()
+
+
+def aeq_frames(rng, lens):
+    return [F.Frame(symbols(rng, n), torch.zeros((n, 4), dtype=torch.int16, device="cuda")) for n in lens]
+
+
+def pdm_frame(rng, n, L=17, state=None):
+    x = torch.from_numpy(rng.integers(-16, 16, (n, 2, 2)).astype(np.int8)).cuda()
+    taps = rng.integers(-32, 32, (L, 2)).astype(np.int8)
+    return F.Frame(x, torch.zeros((F.chain_nsym(n, L), 4), dtype=torch.int16, device="cuda"), taps, state)
+
+
+def run_totals(n, seg, warm):
+    """Runs of a frame of n symbols: how many, their symbols in all, the longest."""
+    if seg <= 0 or seg >= n:
+        return 1, n, n
+    runs = [min(n, k + seg) - max(0, k - warm) for k in range(0, n, seg)]
+    return len(runs), sum(runs), max(runs)
+
+
+@pytest.mark.parametrize("period", [1, 3])
+@pytest.mark.parametrize("na", [32, 64])
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("lens", [[3000], [400] * 250, [400] * 700])
+def test_aeq_route_names_the_kernel_that_runs(lens, kind, na, period):
+    rng = np.random.default_rng(len(lens) + kind)
+    plan = F.Plan(n_aeq=na, alpha_aeq=4080 if na == 64 else 2, mu_shift=9, aeq_update_period=period)
+    plan.set_aeq_kernel(kind)
+    fr = aeq_frames(rng, lens)
+    want = plan.aeq_route(len(lens), sum(lens), max(lens))
+    assert kernels(lambda: F.aeq_run(plan, fr)) == [want]
+    if kind == 0:
+        # few (chain, polarisation) items per SM take the split layout
+        line = 3.5 if na == 64 else 2.8 if period > 1 else 4.0
+        few = 2 * len(lens) < line * torch.cuda.get_device_properties(0).multi_processor_count
+        assert want == ("aeq_split_kernel" if few else "aeq_duo_kernel")
+
+
+@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("n", [5000, 400_000])
+def test_cdc_route_names_the_kernel_that_runs(n, kind):
+    rng = np.random.default_rng(n + kind)
+    plan = F.Plan()
+    plan.set_cdc_kernel(kind)
+    x = torch.from_numpy(rng.integers(-16, 16, (n, 2, 2)).astype(np.int8)).cuda()
+    fr = F.Frame(x, torch.zeros((n, 2, 2), dtype=torch.int16, device="cuda"), np.ones((17, 2), np.int8))
+    items = 2 * -(-(-(-n // 48)) // 32)
+    assert kernels(lambda: F.cdc_run(plan, [fr]))[-1] == plan.cdc_route(items)
+    assert plan.cdc_route(items) == ["cdc_direct_kernel", "cdc_kernel", "cdc_split_kernel"][kind]
