@@ -838,6 +838,23 @@ int64_t single_chains(const SingleFrame &one) {
     return one.seg > 0 ? (one.fr.n_sym + one.seg - 1) / one.seg : 1;
 }
 
+// Symbols of the frame's runs, as its table entries would have them: in all, and of the
+// longest run.  Run k covers k seg .. (k + 1) seg with its warm-up cut at the frame's
+// start; runs grow with k up to the last, which may be short.
+static void single_symbols(const SingleFrame &one, int64_t chains, int64_t &total, int64_t &longest) {
+    const int64_t n = one.fr.n_sym, c = chains;
+    total = longest = n;
+    if (c <= 1) return;
+    auto run = [&](int64_t k) {
+        return std::min(n - k * one.seg, one.seg) + std::min(k * one.seg, one.warmup);
+    };
+    longest = std::max(run(c - 1), run(c - 2));
+    const int64_t cut = std::min(c - 1, one.warmup / one.seg);      // runs 1 .. cut begin at 0
+    const double warm = 0.5 * (double)one.seg * (double)cut * (double)(cut + 1) +
+                        (c - 1 > cut ? (double)(c - 1 - cut) * (double)one.warmup : 0.0);
+    total = n + (int64_t)std::min(warm, 4e18);
+}
+
 fnt_status launch_single(const fnt_plan *p, const SingleFrame &one, int op, cudaStream_t stream, int stages) {
     cudaError_t e = cudaSuccess;
     if ((stages & 1) && op != FNT_OP_AEQ) {
@@ -853,9 +870,9 @@ fnt_status launch_single(const fnt_plan *p, const SingleFrame &one, int op, cuda
             e = cudaMemcpyAsync((void *)one.init, one.fr.state, kStateBytes, cudaMemcpyDeviceToDevice, stream);
             if (e != cudaSuccess) return cuda_fail(e, "copy initial taps");
         }
-        const int64_t longest = one.seg > 0 ? std::min(one.fr.n_sym, one.seg + one.warmup) : one.fr.n_sym;
-        e = aeq_launch_for(p, nullptr, nullptr, (int)chains, one.fr.n_sym + (chains - 1) * one.warmup, longest, stream,
-                           &one);
+        int64_t total, longest;
+        single_symbols(one, chains, total, longest);
+        e = aeq_launch_for(p, nullptr, nullptr, (int)chains, total, longest, stream, &one);
         if (e != cudaSuccess) return cuda_fail(e, "direct aeq kernel launch");
     }
     return FNT_OK;

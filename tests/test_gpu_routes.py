@@ -81,3 +81,25 @@ def test_cdc_route_names_the_kernel_that_runs(n, kind):
     items = 2 * -(-(-(-n // 48)) // 32)
     assert kernels(lambda: F.cdc_run(plan, [fr]))[-1] == plan.cdc_route(items)
     assert plan.cdc_route(items) == ["cdc_direct_kernel", "cdc_kernel", "cdc_split_kernel"][kind]
+
+
+@pytest.mark.parametrize("na", [32, 64])
+@pytest.mark.parametrize("n,seg,warm", [(30000, 512, 0), (30000, 512, 100), (30001, 512, 1 << 20),
+                                        (30001, 512, (1 << 63) - 1), (2600, 512, 3000), (200_000, 250, 4000),
+                                        (511, 512, 1 << 40)])
+def test_one_frame_takes_the_layout_of_its_tables(n, seg, warm, na):
+    """A frame passed as a parameter (a call on it alone, a batch of it) runs in the
+    layout that its runs' lengths give, as it does through tables, also where the
+    warm-up passes the frame's start or seg + warmup passes 64 bits."""
+    rng = np.random.default_rng(n + seg)
+    plan = F.Plan(n_aeq=na, alpha_aeq=4080 if na == 64 else 2, mu_shift=9, aeq_segment=seg, aeq_warmup=warm)
+    f, g = aeq_frames(rng, [n, 1])
+    want = plan.aeq_route(*run_totals(n, seg, warm))
+    assert kernels(lambda: F.aeq_run(plan, [f])) == [want]
+    got = f.out.clone()
+    b = F.Batch(plan, [f], F.OP_AEQ, use_graph=False)
+    assert kernels(b.launch) == [want]
+    assert torch.equal(f.out, got)
+    f.out.zero_()
+    assert kernels(lambda: F.aeq_run(plan, [f, g])) == [want]
+    assert torch.equal(f.out, got)
