@@ -567,8 +567,8 @@ fnt_status build_work(const fnt_plan *p, const fnt_frame_batch *b, int op, Work 
     w.cdc_direct = op != FNT_OP_AEQ && cdc_use_direct(p);
     const bool both = op != FNT_OP_AEQ && !w.cdc_direct && cdc_items_both(p, w);
     w.cdc_both = both;
+    int64_t tiles = 0;
     if (w.cdc_direct) {
-        int64_t tiles = 0;
         for (const DevFrame &df : w.frames) tiles += cdc_direct_tiles(df, op);
         w.cdc_tiles = cdc_direct_tiles_per_item(p, tiles);
     }
@@ -612,9 +612,14 @@ fnt_status build_work(const fnt_plan *p, const fnt_frame_batch *b, int op, Work 
     if (w.items.size() > (size_t)INT32_MAX || w.chains.size() > (size_t)INT32_MAX)
         return fail(FNT_ERR_INVALID, "batch too large");
     // pipelined chunks (chain op only): cut the item list evenly; a chain joins
-    // the first chunk whose CDC items cover everything it reads
+    // the first chunk whose CDC items cover everything it reads.  A chunk is at least
+    // eight transform items or eight direct tiles (a tile holds no more samples than an
+    // item, so a direct batch is cut wherever a transform one is), not eight direct
+    // items, which may be four tiles each.
     int C = 1;
-    if (op == FNT_OP_CHAIN && p->chunks > 1 && (int)w.items.size() >= 8 * p->chunks) C = p->chunks;
+    if (op == FNT_OP_CHAIN && p->chunks > 1 &&
+        (w.cdc_direct ? tiles : (int64_t)w.items.size()) >= 8 * (int64_t)p->chunks)
+        C = p->chunks;
     w.item_cut.assign(C + 1, 0);
     for (int k = 0; k <= C; ++k) w.item_cut[k] = (int)((int64_t)w.items.size() * k / C);
     auto chunk_of = [&](const AeqChain &c) {

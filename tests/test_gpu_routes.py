@@ -103,3 +103,25 @@ def test_one_frame_takes_the_layout_of_its_tables(n, seg, warm, na):
     f.out.zero_()
     assert kernels(lambda: F.aeq_run(plan, [f, g])) == [want]
     assert torch.equal(f.out, got)
+
+
+@pytest.mark.parametrize("n", [20_000, 66_000, 180_000, 400_000])
+@pytest.mark.parametrize("chunks", [2, 16])
+def test_pipeline_cuts_direct_batches_where_it_cuts_transform_ones(n, chunks):
+    """set_pipeline: a batch that the transform CDC runs in chunks is cut in direct
+    form too, with the same results."""
+    rng = np.random.default_rng(n + chunks)
+    counts, outs = [], []
+    f = pdm_frame(rng, n)
+    for kind in (0, 1):
+        plan = F.Plan(mu_shift=9, aeq_segment=512)
+        plan.set_cdc_kernel(kind)
+        plan.set_pipeline(chunks)
+        b = F.Batch(plan, [f], F.OP_CHAIN, use_graph=False)
+        f.out.zero_()
+        b.launch()
+        torch.cuda.synchronize()
+        counts.append(b.kernel_count())
+        outs.append(f.out.clone())
+    assert torch.equal(*outs)
+    assert counts[1] == 2 or counts[0] > 2, counts
