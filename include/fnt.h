@@ -332,7 +332,9 @@ FNT_API fnt_status fnt_plan_set_aeq_occupancy(fnt_plan *plan, int32_t max_warps_
  * FNT_ERR_INVALID outside [0, 2]. */
 FNT_API fnt_status fnt_plan_set_aeq_kernel(fnt_plan *plan, int32_t kind);
 
-/* Picks the CDC kernel of the calls and prepared batches made later with this plan.
+/* Picks the CDC kernel of later launches of this plan (a prepared batch that has
+ * recorded its graph replays what it recorded; one that has not is prepared a second
+ * time, in its next launch, when the choice moves it between 0 and the transforms).
  * 0 (default): the direct form (exact integer dot products; constraint (5) makes
  * the transforms' convolution the same integers).  1 and 2 run the 64-point
  * transforms: 1 = one overlap-save block per lane (each transform in one thread's

@@ -540,31 +540,40 @@ static void add_aeq_chains(const fnt_plan *p, const DevFrame &df, int fi, const 
     }
 }
 
+static fnt_status build_tables(const fnt_plan *p, Work &w, bool direct, int chunks);
+
 fnt_status build_work(const fnt_plan *p, const fnt_frame_batch *b, int op, Work &w) {
     if (!b || b->n_frames < 0 || (b->n_frames > 0 && !b->frames))
         return fail(FNT_ERR_INVALID, "bad frame batch");
     w = Work();
     w.op = op;
     w.frames.resize(b->n_frames);
-    int64_t scratch = 0;
     for (int i = 0; i < b->n_frames; ++i) {
         fnt_status st = make_frame(p, b->frames[i], op, i, w.frames[i]);
         if (st != FNT_OK) return st;
-        if (op == FNT_OP_CHAIN) {
-            w.scratch_off.push_back(scratch);
-            scratch += (w.frames[i].n_sym * 4 + 255) / 256 * 256;
-        }
     }
+    return build_tables(p, w, cdc_use_direct(p), p->chunks);
+}
+
+// The work lists of w.frames, for the direct CDC or the transform kernels.
+static fnt_status build_tables(const fnt_plan *p, Work &w, bool direct, int chunks) {
+    const int op = w.op, n_frames = (int)w.frames.size();
+    int64_t scratch = 0;
+    if (op == FNT_OP_CHAIN)
+        for (const DevFrame &df : w.frames) {
+            w.scratch_off.push_back(scratch);
+            scratch += (df.n_sym * 4 + 255) / 256 * 256;
+        }
     w.scratch_bytes = scratch;
     // Longest frames first, both for their CDC items and their AEQ chains: the
     // serial AEQ recurrences of long frames bound the makespan, and with
     // pipelined chunks they then start in the first chunk.
-    std::vector<int> order(b->n_frames);
-    for (int i = 0; i < b->n_frames; ++i) order[i] = i;
+    std::vector<int> order(n_frames);
+    for (int i = 0; i < n_frames; ++i) order[i] = i;
     if (op == FNT_OP_CHAIN)
         std::stable_sort(order.begin(), order.end(),
                          [&](int a, int c) { return w.frames[a].n_sym > w.frames[c].n_sym; });
-    w.cdc_direct = op != FNT_OP_AEQ && cdc_use_direct(p);
+    w.cdc_direct = op != FNT_OP_AEQ && direct;
     const bool both = op != FNT_OP_AEQ && !w.cdc_direct && cdc_items_both(p, w);
     w.cdc_both = both;
     int64_t tiles = 0;
@@ -617,9 +626,8 @@ fnt_status build_work(const fnt_plan *p, const fnt_frame_batch *b, int op, Work 
     // item, so a direct batch is cut wherever a transform one is), not eight direct
     // items, which may be four tiles each.
     int C = 1;
-    if (op == FNT_OP_CHAIN && p->chunks > 1 &&
-        (w.cdc_direct ? tiles : (int64_t)w.items.size()) >= 8 * (int64_t)p->chunks)
-        C = p->chunks;
+    if (op == FNT_OP_CHAIN && chunks > 1 && (w.cdc_direct ? tiles : (int64_t)w.items.size()) >= 8 * (int64_t)chunks)
+        C = chunks;
     w.item_cut.assign(C + 1, 0);
     for (int k = 0; k <= C; ++k) w.item_cut[k] = (int)((int64_t)w.items.size() * k / C);
     auto chunk_of = [&](const AeqChain &c) {
@@ -1054,8 +1062,17 @@ extern "C" fnt_status fnt_cdc_aeq_run(const fnt_plan *p, const fnt_frame_batch *
 
 struct fnt_batch {
     const fnt_plan *plan = nullptr;
-    Work work;
-    char *dev = nullptr;
+    // The prepared work and its device memory, for the transform CDC (form[0]; also the
+    // AEQ alone) and the direct CDC (form[1]).  One is prepared at creation; the other
+    // when a launch finds that fnt_plan_set_cdc_kernel has picked it since.  A recorded
+    // graph keeps using the form that it was recorded from.
+    struct Form {
+        Work work;
+        char *dev = nullptr;
+    };
+    Form form[2];
+    Form *cur = nullptr;
+    int chunks = 1;                   // the plan's, at creation
     int use_graph = 0;
     cudaGraphExec_t exec = nullptr;
     std::vector<cudaStream_t> side;   // one per pipelined chunk
@@ -1077,9 +1094,75 @@ struct fnt_batch {
     cudaEvent_t in_free = nullptr;    // the previous launch has consumed them
 };
 
+// Lays out and uploads a form whose tables are built (on `stream`, and waits for it).
+static fnt_status prepare_form(fnt_batch *bt, fnt_batch::Form &f, cudaStream_t stream) {
+    Work &w = f.work;
+    layout(w);
+    const size_t C = w.item_cut.size() - 1;
+    // (host inputs may be repointed in the frame table after a graph is captured)
+    w.single = w.frames.size() == 1 && C == 1 && bt->inputs.empty() && (w.op == FNT_OP_AEQ || w.cdc_direct) &&
+               (w.op == FNT_OP_CDC || aeq_use_direct(bt->plan));
+    if (C > 1 && bt->side.empty()) {
+        bt->side.resize(C);
+        bt->ev.resize(2 * C);
+        for (auto &sd : bt->side) cudaStreamCreateWithFlags(&sd, cudaStreamNonBlocking);
+        for (auto &e : bt->ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+    }
+    cudaError_t e = cudaMalloc((void **)&f.dev, w.total);
+    if (e != cudaSuccess) {
+        f.dev = nullptr;
+        return e == cudaErrorMemoryAllocation ? fail(FNT_ERR_NOMEM, "device memory") : cuda_fail(e, "cudaMalloc");
+    }
+    fnt_status st = upload_work(w, f.dev, stream);
+    // the taps of a prepared batch never change: its tap spectra are computed
+    // once here, and its launches (and graph) hold only the CDC and AEQ kernels
+    if (st == FNT_OK) st = launch_spectra(w, f.dev, stream);
+    if (st == FNT_OK) {
+        w.spectra_ready = true;
+        e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) st = cuda_fail(e, "upload sync");
+    }
+    if (st != FNT_OK) {
+        cudaFree(f.dev);
+        f.dev = nullptr;
+    }
+    return st;
+}
+
+// Moves the batch to the form of the CDC that the plan picks now, preparing it on the
+// first such launch.  That may be inside the caller's stream capture, so the set-up runs
+// on a stream of its own with the capture's checks of other calls lifted meanwhile.
+// Frames that are armed by the test hook stay with the transforms.
+static fnt_status match_plan(fnt_batch *bt) {
+    const Work &w = bt->cur->work;
+    if (w.op == FNT_OP_AEQ || w.frames.empty()) return FNT_OK;
+    const bool direct = bt->plan->cdc_kernel == 0 && w.frames[0].flags == 0;
+    if (w.cdc_direct == direct) return FNT_OK;
+    fnt_batch::Form &f = bt->form[direct];
+    if (!f.dev) {
+        f.work = Work();
+        f.work.op = w.op;
+        f.work.frames = w.frames;
+        fnt_status st = build_tables(bt->plan, f.work, direct, bt->chunks);
+        if (st != FNT_OK) return st;
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) return cuda_fail(e, "batch: capture mode");
+        cudaStream_t own = nullptr;
+        e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+        st = e == cudaSuccess ? prepare_form(bt, f, own) : cuda_fail(e, "cudaStreamCreate");
+        if (own) cudaStreamDestroy(own);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (st != FNT_OK) return st;
+    }
+    bt->cur = &f;
+    return FNT_OK;
+}
+
 static fnt_status batch_enqueue(fnt_batch *bt, cudaStream_t stream) {
-    if (bt->side.empty()) return launch_work(bt->plan, bt->work, bt->dev, stream);
-    return launch_pipelined(bt->plan, bt->work, bt->dev, stream, bt->side, bt->ev);
+    const Work &w = bt->cur->work;
+    if (w.item_cut.size() == 2) return launch_work(bt->plan, w, bt->cur->dev, stream);
+    return launch_pipelined(bt->plan, w, bt->cur->dev, stream, bt->side, bt->ev);
 }
 
 // Input copy: the frames' inputs go to the device on the batch's copy stream,
@@ -1107,7 +1190,10 @@ extern "C" fnt_status fnt_batch_create(const fnt_plan *p, const fnt_frame_batch 
     if (!bt) return fail(FNT_ERR_NOMEM, "host memory");
     bt->plan = p;
     bt->use_graph = use_graph;
-    fnt_status st = build_work(p, b, op, bt->work);
+    bt->chunks = p->chunks;
+    bt->cur = &bt->form[op != FNT_OP_AEQ && cdc_use_direct(p)];
+    Work &work = bt->cur->work;
+    fnt_status st = build_work(p, b, op, work);
     if (st != FNT_OK) {
         delete bt;
         return st;
@@ -1116,7 +1202,7 @@ extern "C" fnt_status fnt_batch_create(const fnt_plan *p, const fnt_frame_batch 
         // page-locked host buffers are used in place through their device
         // mapping; the prepared work cannot stage pageable ones
         for (int i = 0; i < b->n_frames; ++i) {
-            DevFrame &df = bt->work.frames[i];
+            DevFrame &df = work.frames[i];
             if (df.n == 0) continue;
             void *vin = device_view(b->frames[i].in), *vout = device_view(b->frames[i].out);
             if (!vin || !vout) {
@@ -1129,32 +1215,10 @@ extern "C" fnt_status fnt_batch_create(const fnt_plan *p, const fnt_frame_batch 
             bt->inputs.push_back({i, b->frames[i].in, vin, 0, in_bytes(b->frames[i], op)});
         }
     }
-    layout(bt->work);
-    const int C = (int)bt->work.item_cut.size() - 1;
-    // (host inputs may be repointed in the frame table after a graph is captured)
-    bt->work.single = bt->work.frames.size() == 1 && C == 1 && bt->inputs.empty() && single_direct(p, op);
-    if (C > 1) {
-        bt->side.resize(C);
-        bt->ev.resize(2 * C);
-        for (auto &sd : bt->side) cudaStreamCreateWithFlags(&sd, cudaStreamNonBlocking);
-        for (auto &e : bt->ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
-    }
-    cudaError_t e = cudaMalloc((void **)&bt->dev, bt->work.total);
-    if (e != cudaSuccess) {
-        delete bt;
-        return e == cudaErrorMemoryAllocation ? fail(FNT_ERR_NOMEM, "device memory") : cuda_fail(e, "cudaMalloc");
-    }
-    st = upload_work(bt->work, bt->dev, 0);
-    // the taps of a prepared batch never change: its tap spectra are computed
-    // once here, and its launches (and graph) hold only the CDC and AEQ kernels
-    if (st == FNT_OK) st = launch_spectra(bt->work, bt->dev, 0);
-    if (st == FNT_OK) {
-        bt->work.spectra_ready = true;
-        e = cudaStreamSynchronize(0);
-        if (e != cudaSuccess) st = cuda_fail(e, "upload sync");
-    }
+    st = prepare_form(bt, *bt->cur, 0);
     if (st != FNT_OK) {
-        cudaFree(bt->dev);
+        for (auto &sd : bt->side) cudaStreamDestroy(sd);
+        for (auto &e : bt->ev) cudaEventDestroy(e);
         delete bt;
         return st;
     }
@@ -1183,15 +1247,18 @@ extern "C" fnt_status fnt_batch_set_input_copy(fnt_batch *bt, int32_t on) {
     if (e != cudaSuccess) return cuda_fail(e, "input copy");
     // the kernels read the frame table from device memory: repoint the inputs
     // there (a captured graph stays valid)
-    for (const fnt_batch::Input &in : bt->inputs) {
-        DevFrame &df = bt->work.frames[in.frame];
-        const int8_t *p = on ? (const int8_t *)(bt->dev_in + in.off) : (const int8_t *)in.view;
-        df.in = p;
-        if (bt->work.op == FNT_OP_AEQ) df.aeq_in = (int8_t *)p;
+    for (fnt_batch::Form &f : bt->form) {
+        if (!f.dev) continue;
+        for (const fnt_batch::Input &in : bt->inputs) {
+            DevFrame &df = f.work.frames[in.frame];
+            const int8_t *p = on ? (const int8_t *)(bt->dev_in + in.off) : (const int8_t *)in.view;
+            df.in = p;
+            if (f.work.op == FNT_OP_AEQ) df.aeq_in = (int8_t *)p;
+        }
+        e = cudaMemcpy(f.dev + f.work.off_frames, f.work.frames.data(), f.work.frames.size() * sizeof(DevFrame),
+                       cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_fail(e, "input copy: frame table");
     }
-    e = cudaMemcpy(bt->dev + bt->work.off_frames, bt->work.frames.data(), bt->work.frames.size() * sizeof(DevFrame),
-                   cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(e, "input copy: frame table");
     bt->in_copy = on != 0;
     return FNT_OK;
 }
@@ -1213,6 +1280,10 @@ extern "C" fnt_status fnt_batch_launch(fnt_batch *bt, void *stream_) {
 }
 
 static fnt_status batch_launch_all(fnt_batch *bt, cudaStream_t stream) {
+    if (!bt->exec) {
+        fnt_status st = match_plan(bt);
+        if (st != FNT_OK) return st;
+    }
     if (!bt->use_graph) return batch_enqueue(bt, stream);
     if (!bt->exec) {
         cudaStream_t cap;
@@ -1247,9 +1318,11 @@ extern "C" fnt_status fnt_batch_launch_stage(fnt_batch *bt, int32_t stage, void 
     if (stage != 0 && stage != 1) return fail(FNT_ERR_INVALID, "stage must be 0 (CDC) or 1 (AEQ)");
     cudaStream_t stream = (cudaStream_t)stream_;
     // with the input copy on, the stage that reads the inputs copies them first
-    const bool reads_input = bt->in_copy && stage == (bt->work.op == FNT_OP_AEQ ? 1 : 0);
-    fnt_status st = reads_input ? start_input_copy(bt, stream) : FNT_OK;
-    if (st == FNT_OK) st = launch_work(bt->plan, bt->work, bt->dev, stream, 1 << stage);
+    const bool reads_input = bt->in_copy && stage == (bt->cur->work.op == FNT_OP_AEQ ? 1 : 0);
+    // (the AEQ stage reads what the last CDC stage wrote, wherever that was)
+    fnt_status st = stage == 0 ? match_plan(bt) : FNT_OK;
+    if (st == FNT_OK && reads_input) st = start_input_copy(bt, stream);
+    if (st == FNT_OK) st = launch_work(bt->plan, bt->cur->work, bt->cur->dev, stream, 1 << stage);
     if (st == FNT_OK && reads_input) {
         cudaError_t e = cudaEventRecord(bt->in_free, stream);
         if (e != cudaSuccess) st = cuda_fail(e, "batch input release");
@@ -1257,7 +1330,7 @@ extern "C" fnt_status fnt_batch_launch_stage(fnt_batch *bt, int32_t stage, void 
     return st;
 }
 
-extern "C" int32_t fnt_batch_kernel_count(const fnt_batch *bt) { return bt ? work_kernel_count(bt->work) : 0; }
+extern "C" int32_t fnt_batch_kernel_count(const fnt_batch *bt) { return bt ? work_kernel_count(bt->cur->work) : 0; }
 
 extern "C" fnt_status fnt_batch_destroy(fnt_batch *bt) {
     if (!bt) return FNT_OK;
@@ -1269,7 +1342,7 @@ extern "C" fnt_status fnt_batch_destroy(fnt_batch *bt) {
     if (bt->copy_done) cudaEventDestroy(bt->copy_done);
     if (bt->in_free) cudaEventDestroy(bt->in_free);
     cudaFree(bt->dev_in);
-    cudaFree(bt->dev);
+    for (auto &f : bt->form) cudaFree(f.dev);
     delete bt;
     return FNT_OK;
 }

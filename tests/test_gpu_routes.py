@@ -125,3 +125,78 @@ def test_pipeline_cuts_direct_batches_where_it_cuts_transform_ones(n, chunks):
         outs.append(f.out.clone())
     assert torch.equal(*outs)
     assert counts[1] == 2 or counts[0] > 2, counts
+
+
+CDC_NAMES = ["cdc_direct_kernel", "cdc_kernel", "cdc_split_kernel"]
+
+
+@pytest.mark.parametrize("chunks", [1, 4])
+@pytest.mark.parametrize("lens", [[30_000], [9000, 0, 517, 40_000]])
+@pytest.mark.parametrize("first", [0, 1, 2])
+def test_prepared_batch_follows_the_cdc_kernel(lens, first, chunks):
+    """set_cdc_kernel acts on the next launch of an existing batch (whole, by stage or
+    captured by the caller), until the batch has recorded a graph of its own."""
+    rng = np.random.default_rng(sum(lens) + first)
+    plan = F.Plan(mu_shift=9, aeq_segment=512)
+    plan.set_pipeline(chunks)
+    frames = [pdm_frame(rng, n, L) for n, L in zip(lens, (17, 5, 31, 8))]
+    F.cdc_aeq_run(plan, frames)
+    torch.cuda.synchronize()
+    want = [f.out.clone() for f in frames]
+    plan.set_cdc_kernel(first)
+    b = F.Batch(plan, frames, F.OP_CHAIN, use_graph=False)
+    g = F.Batch(plan, frames, F.OP_CHAIN, use_graph=True)
+
+    def check(names, kind):
+        # (preparing the transform form also computes the tap spectra)
+        assert {k for k in names if k.startswith("cdc")} - {"cdc_spectra_kernel"} == {CDC_NAMES[kind]}
+        assert all(torch.equal(f.out, w) for f, w in zip(frames, want)), kind
+        for f in frames:
+            f.out.zero_()
+
+    def stages():
+        b.launch_stage(0)
+        b.launch_stage(1)
+
+    for kind in (first, 1, 0, 2, 0, 1):
+        plan.set_cdc_kernel(kind)
+        check(kernels(b.launch), kind)
+        check(kernels(stages), kind)
+    # the caller's capture, on a batch that was made in the other form
+    plan.set_cdc_kernel(0 if first else 1)
+    c = F.Batch(plan, frames, F.OP_CHAIN, use_graph=False)
+    plan.set_cdc_kernel(first)
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=side):
+        c.launch(side)
+    check(kernels(graph.replay), first)
+    # a recorded graph stays as it is
+    plan.set_cdc_kernel(2 - first)
+    check(kernels(g.launch), 2 - first)
+    plan.set_cdc_kernel(first)
+    check(kernels(g.launch), 2 - first)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("op", [F.OP_CDC, F.OP_CHAIN])
+def test_input_copy_in_both_forms_of_a_batch(op, graph):
+    """Host inputs read in place or through the batch's copy, in the form the batch was
+    made in and in the one it moved to."""
+    rng = np.random.default_rng(op)
+    plan = F.Plan(mu_shift=9)
+    xs = [torch.from_numpy(rng.integers(-16, 16, (n, 2, 2)).astype(np.int8)).pin_memory() for n in (5000, 700)]
+    taps = rng.integers(-32, 32, (17, 2)).astype(np.int8)
+    shapes = [(x.shape[0], 2, 2) if op == F.OP_CDC else (F.chain_nsym(x.shape[0], 17), 4) for x in xs]
+    outs = [torch.zeros(s, dtype=torch.int16).pin_memory() for s in shapes]
+    dev = [F.Frame(x.cuda(), torch.zeros(s, dtype=torch.int16, device="cuda"), taps) for x, s in zip(xs, shapes)]
+    (F.cdc_run if op == F.OP_CDC else F.cdc_aeq_run)(plan, dev)
+    want = [f.out.cpu() for f in dev]
+    b = F.Batch(plan, [F.Frame(x, o, taps) for x, o in zip(xs, outs)], op, use_graph=graph, host=True)
+    for kind, copy in [(0, False), (1, False), (1, True), (0, True), (0, False), (1, False)]:
+        plan.set_cdc_kernel(kind)
+        b.set_input_copy(copy)
+        for o in outs:
+            o.zero_()
+        b.launch()
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, w) for o, w in zip(outs, want)), (kind, copy)
