@@ -307,7 +307,8 @@ def run_fnt(args, rank, world, local_rank, oracle_pool=None):
         p = fnt.Plan(n_aeq=wl["n_aeq"], alpha_aeq=wl["alpha_aeq"], mu_shift=MU_SHIFT, aeq_segment=segment,
                      aeq_warmup=warmup, aeq_update_period=wl.get("period", 1), aeq_freq_sum=wl.get("freq_sum", 0))
         p.set_tensor_gradient(args.tensor_gradient)
-        p.set_aeq_kernel(args.aeq_kernel)
+        # (the tensor-core gradient is transform kernel 1's)
+        p.set_aeq_kernel(1 if args.tensor_gradient and args.aeq_kernel == 0 else args.aeq_kernel)
         p.set_cdc_kernel(args.cdc_kernel)
         return p
 
@@ -1041,7 +1042,8 @@ def main(argv=None):
                     help="cfg2 / cfg5: AEQ kernel (0 direct form, 1 transforms, a warp, 2 transforms, a CTA per chain "
                          "and polarisation)")
     ap.add_argument("--tensor-gradient", action="store_true",
-                    help="cfg2 / cfg5: AEQ gradient on the tensor cores (bit-identical; off = integer path)")
+                    help="cfg2 / cfg5: AEQ gradient on the tensor cores, in transform kernel 1 unless --aeq-kernel "
+                         "says otherwise (bit-identical; off = integer path)")
     ap.add_argument("--aeq-freq-sum", type=int, default=0, choices=(0, 1, 2),
                     help="cfg2 / cfg5: AEQ inputs summed in Z_F before the inverse transform (1 literal, 2 guarded)")
     ap.add_argument("--aeq-period", type=int, default=1,

@@ -254,7 +254,8 @@ typedef struct fnt_batch fnt_batch;
  * above, and change no result.
  *
  * Prepares a batch once for repeated launches: validates it, builds the work
- * lists (frames split into 32-block CDC items; AEQ chains or segments sorted
+ * lists (frames split into CDC items: up to four tiles of 256 outputs each in
+ * direct form, 32 blocks for the transform kernels; AEQ chains or segments sorted
  * longest first), uploads them and allocates the intermediate buffers, all in
  * device memory owned by the fnt_batch.  Buffers are device memory
  * (host_buffers = 0) or page-locked host memory (host_buffers = 1), which the
@@ -296,8 +297,9 @@ FNT_API int32_t fnt_batch_kernel_count(const fnt_batch *b);
 FNT_API fnt_status fnt_batch_destroy(fnt_batch *b);
 
 /* Sets the warps per CTA of the transform CDC and AEQ kernels in later launches of
- * this plan (autotuner hook; the direct forms have their own).  0 keeps the current
- * value. */
+ * this plan (autotuner hook).  0 keeps the current value.  It has no effect on the
+ * direct forms, which run unless fnt_plan_set_cdc_kernel or fnt_plan_set_aeq_kernel
+ * picks a transform kernel (AEQ kernel 2 has its own CTA size too). */
 FNT_API fnt_status fnt_plan_set_launch(fnt_plan *plan, int32_t cdc_warps, int32_t aeq_warps);
 
 /* Prepared chain batches created after this call split their work into
@@ -311,8 +313,9 @@ FNT_API fnt_status fnt_plan_set_pipeline(fnt_plan *plan, int32_t chunks);
 /* Caps the AEQ warps resident per SM for later launches of this plan
  * (autotuner hook): each AEQ CTA then reserves enough shared memory that at
  * most max(1, max_warps_per_sm / aeq warps per CTA) CTAs share an SM.  0
- * (default) lets resources decide (transform kernels only, see
- * fnt_plan_set_aeq_kernel).  Long serial AEQ chains (frames with fresh
+ * (default) lets resources decide.  It applies to the transform AEQ kernel 1 and
+ * has no effect on the direct form, which runs unless fnt_plan_set_aeq_kernel picks
+ * that kernel.  Long serial AEQ chains (frames with fresh
  * taps and no segments) finish sooner when fewer share an SM, which can
  * shorten a batch whose longest chain sets its time.  Results do not depend on
  * it.  FNT_ERR_INVALID outside [0, 64]. */
@@ -328,7 +331,7 @@ FNT_API fnt_status fnt_plan_set_aeq_occupancy(fnt_plan *plan, int32_t max_warps_
  * over 288 threads and cuts the time per block of a lone chain.  Plans with
  * aeq_freq_sum != 0 run 1 where 2 is asked for.  Results do not depend on it for
  * samples and taps inside the ranges stated above.  The warps per CTA, the occupancy
- * cap and the tensor-core gradient set on a plan apply to kernels 1 and 2.
+ * cap and the tensor-core gradient set on a plan apply to kernel 1 only.
  * FNT_ERR_INVALID outside [0, 2]. */
 FNT_API fnt_status fnt_plan_set_aeq_kernel(fnt_plan *plan, int32_t kind);
 
@@ -343,7 +346,7 @@ FNT_API fnt_status fnt_plan_set_aeq_kernel(fnt_plan *plan, int32_t kind);
  * "Fermat number transform"), for work too small to fill the GPU one block per
  * lane.  Results do not depend on it for samples and taps inside the ranges stated
  * above.  The warps per CTA and polarisations per item set on a plan apply to
- * kernels 1 and 2.  FNT_ERR_INVALID outside [0, 2]. */
+ * kernels 1 and 2 only.  FNT_ERR_INVALID outside [0, 2]. */
 FNT_API fnt_status fnt_plan_set_cdc_kernel(fnt_plan *plan, int32_t kind);
 
 /* The one-block-per-lane CDC kernel fetches the 32 input windows of a PDM work
@@ -393,12 +396,16 @@ FNT_API fnt_status fnt_plan_initial_taps(const fnt_plan *plan, int32_t *state);
 /* CDC work items created after this call cover 32 overlap-save blocks of one
  * polarisation (pols = 1) or of both polarisations of a PDM frame (pols = 2);
  * 0 (default) picks 2 when the work fills the GPU at least twice over and 1
- * otherwise.  Results do not depend on it. */
+ * otherwise.  The items are the transform kernels': the direct form, which runs
+ * unless fnt_plan_set_cdc_kernel picks one of them, takes all polarisations of a
+ * tile whatever is set here.  Results do not depend on it. */
 FNT_API fnt_status fnt_plan_set_cdc_items(fnt_plan *plan, int32_t pols);
 
-/* on = 1: later AEQ launches of this plan compute the gradient of eq. (6) on the
- * tensor cores instead of the integer pipes (default 0).  Results are
- * bit-identical: e z (|e z| <= 2^46) is split into four balanced 12-bit limbs,
+/* on = 1: later launches of the transform AEQ kernel 1 with this plan compute the
+ * gradient of eq. (6) on the tensor cores instead of the integer pipes (default 0).
+ * Pick that kernel with fnt_plan_set_aeq_kernel(plan, 1): the direct form, which
+ * runs by default and is faster, and kernel 2 form the gradient on the integer pipes
+ * whatever is set here.  Results are bit-identical: e z (|e z| <= 2^46) is split into four balanced 12-bit limbs,
  * which, like the 5-bit input, are exact in f16, and every per-block sum of
  * limb x input products stays below 2^24, so the f32 accumulation is exact and
  * the limb sums are recombined in int64.  Off by default because the paper's

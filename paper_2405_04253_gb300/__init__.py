@@ -219,13 +219,16 @@ class Plan:
             pass
 
     def set_launch(self, cdc_warps: int = 0, aeq_warps: int = 0):
+        """Warps per CTA of the transform kernels (0 = keep); no effect on the direct
+        forms, which run unless set_cdc_kernel / set_aeq_kernel pick a transform kernel."""
         check(lib().fnt_plan_set_launch(self.handle, cdc_warps, aeq_warps))
 
     def set_pipeline(self, chunks: int):
         check(lib().fnt_plan_set_pipeline(self.handle, chunks))
 
     def set_aeq_occupancy(self, max_warps_per_sm: int):
-        """Caps the AEQ warps resident per SM (0 = no cap); same results."""
+        """Caps the warps of AEQ kernel 1 resident per SM (0 = no cap); same results.
+        No effect on the direct form: pick the kernel with set_aeq_kernel(1)."""
         check(lib().fnt_plan_set_aeq_occupancy(self.handle, int(max_warps_per_sm)))
 
     def set_aeq_kernel(self, kind: int):
@@ -270,11 +273,13 @@ class Plan:
         return st
 
     def set_cdc_items(self, pols: int):
-        """CDC items of one (1) or both (2) polarisations; 0 = automatic."""
+        """Transform CDC items of one (1) or both (2) polarisations; 0 = automatic.
+        No effect on the direct form: pick a transform kernel with set_cdc_kernel."""
         check(lib().fnt_plan_set_cdc_items(self.handle, pols))
 
     def set_tensor_gradient(self, on: bool):
-        """AEQ gradient on the tensor cores (exact; same results)."""
+        """Gradient of AEQ kernel 1 on the tensor cores (exact; same results).  No
+        effect on the direct form: pick the kernel with set_aeq_kernel(1)."""
         check(lib().fnt_plan_set_tensor_gradient(self.handle, int(bool(on))))
 
 

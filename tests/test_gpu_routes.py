@@ -16,8 +16,9 @@ if not torch.cuda.is_available():
 import paper_2405_04253_gb300 as F  # noqa: E402
 
 
-def kernels(fn):
-    """Names of the library's kernels that fn launches, in order of their start."""
+def kernels(fn, instance=False):
+    """Names of the library's kernels that fn launches, in order of their start
+    (instance: with their template arguments)."""
     from torch.profiler import ProfilerActivity, profile
     for _ in range(3):                       # the first session of a process may record nothing
         torch.cuda.synchronize()
@@ -26,7 +27,8 @@ def kernels(fn):
             torch.cuda.synchronize()
         ev = sorted((e for e in prof.events() if "fnt::" in e.name), key=lambda e: e.time_range.start)
         if ev:
-            return [re.search(r"::(\w+)[<(]", e.name.replace("(anonymous namespace)::", "")).group(1) for e in ev]
+            pat = r"::(\w+(?:<[^(]*>)?)\(" if instance else r"::(\w+)[<(]"
+            return [re.search(pat, e.name.replace("(anonymous namespace)::", "")).group(1) for e in ev]
     pytest.skip("the CUDA profiler records no kernels here")
 
 
@@ -200,3 +202,28 @@ def test_input_copy_in_both_forms_of_a_batch(op, graph):
         b.launch()
         torch.cuda.synchronize()
         assert all(torch.equal(o, w) for o, w in zip(outs, want)), (kind, copy)
+
+
+def test_transform_settings_act_on_the_kernel_that_has_them():
+    """The tensor-core gradient and two-polarisation CDC items change the instance of
+    the transform kernels that runs; the direct forms ignore them."""
+    rng = np.random.default_rng(5)
+    f = pdm_frame(rng, 30_000)
+
+    def instances(kind, tensor, pols):
+        plan = F.Plan(mu_shift=9, aeq_segment=512)
+        plan.set_aeq_kernel(kind)
+        plan.set_cdc_kernel(kind)
+        plan.set_tensor_gradient(tensor)
+        plan.set_cdc_items(pols)
+        f.out.zero_()
+        names = kernels(lambda: F.cdc_aeq_run(plan, [f]), instance=True)
+        return names[-2:], f.out.clone()
+
+    base, want = instances(1, False, 1)
+    tensor, got = instances(1, True, 2)
+    assert base[0] != tensor[0] and base[1] != tensor[1] and torch.equal(got, want)
+    assert [n.split("<")[0] for n in base] == ["cdc_kernel", "aeq_kernel"] == [n.split("<")[0] for n in tensor]
+    direct, got = instances(0, True, 2)
+    assert direct == instances(0, False, 1)[0] and torch.equal(got, want)
+    assert [n.split("<")[0] for n in direct] == ["cdc_direct_kernel", "aeq_split_kernel"]
