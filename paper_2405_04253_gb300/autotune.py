@@ -1,17 +1,21 @@
-"""Launch-shape autotuner for libfnt.
+"""Launch-shape autotuner for libfnt's transform kernels.
 
 Times each candidate (CDC warps per CTA; AEQ warps per CTA with a cap on the
 AEQ warps resident per SM) on a prepared batch with CUDA events around each
-stage on the launching stream, after warm-up, and keeps the fastest per stage.  Results are cached in a JSON file keyed by
-the workload's shape, so a later run with the same shape reuses them.  Only
-launch shapes change: results are bit-identical for every candidate.
+stage on the launching stream, after warm-up, and keeps the fastest per stage.
+Only stages whose kernel has these settings are tuned: the direct forms, which a
+plan runs unless it picks a transform kernel, have shapes of their own, and so have
+the kernels that a plan picks with set_cdc_kernel(2) and set_aeq_kernel(2).  Results
+are cached in a JSON file keyed by the workload's shape and the tuned stages, so a
+later run with the same shape reuses them.  Only launch shapes change: results are
+bit-identical for every candidate.
 """
 from __future__ import annotations
 
 import json
 import os
 
-from . import OP_CHAIN, Batch, Plan
+from . import OP_AEQ, OP_CDC, OP_CHAIN, Batch, Plan
 
 CANDIDATES = (1, 2, 3, 4)
 _SRC_TAG = None
@@ -33,12 +37,24 @@ def _src_tag() -> str:
 OCCUPANCY = (0, 12, 16, 20)          # AEQ warps per SM cap (0: none)
 
 
-def _key(plan: Plan, frames, op: int) -> str:
+def tunable(plan: Plan, op: int) -> tuple:
+    """The stages of `op` ("cdc", "aeq") whose kernels have launch settings."""
+    stages = []
+    # asked for work that fills the GPU: smaller work may take another transform kernel
+    # (also on a plan that picks none: aeq_freq_sum = 1)
+    if op != OP_AEQ and plan.cdc_route(1 << 20) == "cdc_kernel":
+        stages.append("cdc")
+    if op != OP_CDC and plan.aeq_route(1 << 20, 1 << 20, 1) == "aeq_kernel":
+        stages.append("aeq")
+    return tuple(stages)
+
+
+def _key(plan: Plan, frames, op: int, stages=("cdc", "aeq")) -> str:
     d = plan.desc
     lens = sorted(int(f.n) for f in frames)
     total = sum(lens)
     return (f"op{op}_n{len(frames)}_tot{total}_max{lens[-1] if lens else 0}_aeq{d.n_aeq}"
-            f"_seg{d.aeq_segment}_{d.aeq_warmup}_p{d.aeq_update_period}_src{_src_tag()}")
+            f"_seg{d.aeq_segment}_{d.aeq_warmup}_p{d.aeq_update_period}_{'_'.join(stages)}_src{_src_tag()}")
 
 
 def _time_stage(batch: Batch, stage: int, reps: int, stream) -> float:
@@ -54,27 +70,39 @@ def _time_stage(batch: Batch, stage: int, reps: int, stream) -> float:
     return evs[0].elapsed_time(evs[1]) / reps
 
 
+def _apply(plan: Plan, best: dict):
+    if "cdc" in best["tuned"]:
+        plan.set_launch(cdc_warps=best["cdc_warps"])
+    if "aeq" in best["tuned"]:
+        plan.set_launch(aeq_warps=best["aeq_warps"])
+        plan.set_aeq_occupancy(best["aeq_occupancy"])
+
+
 def tune(plan: Plan, frames, op: int = OP_CHAIN, reps: int = 20, cache: str | None = None) -> dict:
     """Picks and applies the fastest launch shape for each stage of `op` on
-    these frames; returns {"cdc_warps", "aeq_warps", "aeq_occupancy", "cdc_ms",
-    "aeq_ms"}."""
+    these frames that can be tuned; returns {"tuned": those stages, "cdc_warps",
+    "aeq_warps", "aeq_occupancy", "cdc_ms", "aeq_ms"}.  A stage that cannot be tuned
+    is timed once, as it runs, and the plan's settings for it are left alone."""
     import torch
-    key = _key(plan, frames, op)
-    if cache and os.path.exists(cache):
+    stages = tunable(plan, op)
+    key = _key(plan, frames, op, stages)
+    if cache and stages and os.path.exists(cache):
         try:
             with open(cache) as fh:
                 hit = json.load(fh).get(key)
         except (OSError, ValueError):
             hit = None
         if hit:
-            plan.set_launch(hit["cdc_warps"], hit["aeq_warps"])
-            plan.set_aeq_occupancy(hit.get("aeq_occupancy", 0))
+            _apply(plan, hit)
             return hit
     stream = torch.cuda.current_stream()
     batch = Batch(plan, frames, op, use_graph=False)
-    best = {}
+    best = {"tuned": list(stages), "cdc_warps": 4, "aeq_warps": 2, "aeq_occupancy": 0}
     for stage, name in ((0, "cdc"), (1, "aeq")):
-        if stage == 0 and op == 1 or stage == 1 and op == 0:
+        if op == (OP_AEQ, OP_CDC)[stage]:
+            continue
+        if name not in stages:
+            best[name + "_ms"] = _time_stage(batch, stage, reps, stream)
             continue
         for w in CANDIDATES:
             for occ in (OCCUPANCY if stage == 1 else (0,)):
@@ -91,13 +119,9 @@ def tune(plan: Plan, frames, op: int = OP_CHAIN, reps: int = 20, cache: str | No
                     best[name + "_warps"] = w
                     if stage == 1:
                         best["aeq_occupancy"] = occ
-    best.setdefault("cdc_warps", 4)
-    best.setdefault("aeq_warps", 2)
-    best.setdefault("aeq_occupancy", 0)
-    plan.set_launch(best["cdc_warps"], best["aeq_warps"])
-    plan.set_aeq_occupancy(best["aeq_occupancy"])
+    _apply(plan, best)
     batch.close()
-    if cache:
+    if cache and stages:
         data = {}
         if os.path.exists(cache):
             try:
