@@ -184,8 +184,10 @@ FNT_API fnt_status fnt_op_counts_for(const fnt_plan_desc *desc, int32_t cd_len, 
  *   cd_taps   HOST int8 [cd_len][2] (re, im), 6-bit signed [-32, 31]; CDC and
  *             chain only (ignored by the AEQ alone).
  *   aeq_state DEVICE int32 [4 (S2)][4 (S1)][K] master taps of the AEQ
- *             (tap = state >> 16), read at the start and overwritten with the
- *             adapted taps at the end; NULL = start from the plan's initial taps
+ *             (tap = state >> 16, a 14-bit tap: the update keeps every state in
+ *             [-2^29, 2^29), and results are defined for states that start
+ *             there), read at the start and overwritten with the adapted taps at
+ *             the end; NULL = start from the plan's initial taps
  *             and keep nothing.  With AEQ segments every segment starts from the
  *             state as it was when the call began (the library copies it first)
  *             and the state then receives the final taps of the last segment.
@@ -366,7 +368,8 @@ FNT_API fnt_status fnt_plan_set_cdc_kernel(fnt_plan *plan, int32_t kind);
 FNT_API fnt_status fnt_device_faults(int32_t clear, uint32_t *faults);
 
 /* Test hook: with mode 1, later one-shot calls and prepared batches of this
- * plan arm the CDC's window barrier without issuing the bulk copy, so the
+ * plan run the transform CDC (the direct form has no such wait) and arm its window
+ * barrier without issuing the bulk copy, so the
  * bounded wait runs out and sets FNT_FAULT_CDC_WINDOW_WAIT: a way to test that
  * path without faulting anything.  0 (default) is normal operation.
  * FNT_ERR_INVALID for other modes. */
@@ -405,11 +408,11 @@ FNT_API fnt_status fnt_plan_set_cdc_items(fnt_plan *plan, int32_t pols);
  * gradient of eq. (6) on the tensor cores instead of the integer pipes (default 0).
  * Pick that kernel with fnt_plan_set_aeq_kernel(plan, 1): the direct form, which
  * runs by default and is faster, and kernel 2 form the gradient on the integer pipes
- * whatever is set here.  Results are bit-identical: e z (|e z| <= 2^46) is split into four balanced 12-bit limbs,
- * which, like the 5-bit input, are exact in f16, and every per-block sum of
- * limb x input products stays below 2^24, so the f32 accumulation is exact and
- * the limb sums are recombined in int64.  Off by default because the paper's
- * path is integer arithmetic throughout. */
+ * whatever is set here.  Results are bit-identical: e z (|e z| <= 2^46) is split
+ * into four balanced 12-bit limbs, which, like the 5-bit input, are exact in f16, and
+ * every per-block sum of limb x input products stays below 2^24, so the f32
+ * accumulation is exact and the limb sums are recombined in int64.  Off by default
+ * because the paper's path is integer arithmetic throughout. */
 FNT_API fnt_status fnt_plan_set_tensor_gradient(fnt_plan *plan, int32_t on);
 
 /* ------------------------------------------------- allocation-free chain ---- */
@@ -432,9 +435,11 @@ FNT_API fnt_status fnt_plan_set_tensor_gradient(fnt_plan *plan, int32_t on);
  * first call on a device, with that device current, sets up: it looks up the
  * array's address, creates the events that guard the library's host copies of
  * the work tables, and (once per process) page-locks those host copies; make
- * that first call outside any stream capture.  Each call uploads its tables
- * with one asynchronous copy and does not wait for the stream (a host copy is
- * reused four calls later, after its last upload has run).  The call cannot be
+ * that first call outside any stream capture.  In direct form a call has no tables:
+ * its kernels take the frame as a parameter.  With a transform kernel picked for
+ * either stage each call uploads its tables with one asynchronous copy.  No call
+ * waits for the stream (a host copy is reused four table calls later, after its last
+ * upload has run).  The call cannot be
  * captured in a CUDA graph: on a capturing stream it returns FNT_ERR_INVALID
  * and enqueues nothing.  All calls on a device share the array and overwrite
  * it, so calls whose work overlaps on the GPU race: keep them on one stream or

@@ -231,13 +231,14 @@ __device__ __forceinline__ int32_t out_of(int32_t y) { return min(max(y >> 7, -3
 // at N = 64 for a lone chain (0.60 and 0.83 us with the transforms on a CTA); with a
 // whole block in one warp it was 0.34 and 0.61 us, about 200 and 500 dependent
 // instructions at 3 to 4 cycles each.  The launch bound of four CTAs an SM (64
-// registers at N = 64) lets four items share an SM and takes 8 to 10 % off a block
-// against no bound; a bound of two or three gives less, five and six cost time.
+// registers at N = 64) lets four items share an SM and takes 9 % (N = 32) and 7 % off a
+// block of a lone chain against no bound (0.2078, 0.2885 us against 0.2278, 0.3092); a
+// bound of two gives less (0.2117, 0.3029), five and six cost time.
 template <int NA>
 struct SplitCfg {
-    // batches of 16 (N = 32) and 8 blocks: half that costs 2.5 % of a block, twice
-    // that more again (0.228, 0.325 us against 0.234, 0.333 and 0.251, 0.338, before
-    // the launch bound)
+    // batches of 16 (N = 32) and 8 blocks: with half that a block of a lone chain takes
+    // 0.2139 and 0.3061 us, not 0.2078 and 0.2885; twice that takes 0.2057 us at N = 32
+    // and passes the static shared memory at N = 64
     using C = DirCfg<NA, NA == 64 ? 8 : 16>;
     static constexpr int NC = (NA - kAeqK) / 16;          // output warps
     static constexpr int NGW = 4;                         // gradient warps

@@ -266,14 +266,14 @@ size_t fnt::aeq_min_smem(const fnt_plan *p) {
 
 extern "C" fnt_status fnt_plan_set_aeq_kernel(fnt_plan *p, int32_t kind) {
     if (!p) return fail(FNT_ERR_INVALID, "null plan");
-    if (kind < 0 || kind > 2) return fail(FNT_ERR_INVALID, "AEQ kernel must be 0 (auto), 1 or 2");
+    if (kind < 0 || kind > 2) return fail(FNT_ERR_INVALID, "AEQ kernel must be 0 (direct form), 1 or 2");
     p->aeq_kernel = kind;
     return FNT_OK;
 }
 
 extern "C" fnt_status fnt_plan_set_cdc_kernel(fnt_plan *p, int32_t kind) {
     if (!p) return fail(FNT_ERR_INVALID, "null plan");
-    if (kind < 0 || kind > 2) return fail(FNT_ERR_INVALID, "CDC kernel must be 0 (auto), 1 or 2");
+    if (kind < 0 || kind > 2) return fail(FNT_ERR_INVALID, "CDC kernel must be 0 (direct form), 1 or 2");
     p->cdc_kernel = kind;
     return FNT_OK;
 }

@@ -22,7 +22,7 @@
 // between tap groups.
 //
 // Bound: dp4a issue (40 a PDM sample at L = 19 against 12 bytes moved, about equal to
-// the HBM time) for the CDC: 2^24 PDM samples, 19 taps in 53 us, 3.8 TB/s (245 us with
+// the HBM time) for the CDC: 2^24 PDM samples, 19 taps in 51 us, 3.9 TB/s (245 us with
 // the transforms).  Latency for small frames.
 #include <algorithm>
 

@@ -22,8 +22,8 @@ struct fnt_plan {
     int tensor_gradient = 0;     // AEQ gradient on the tensor cores (opt-in, same results)
     int cdc_pols_per_item = 0;   // CDC items: 0 auto, 1 one polarisation, 2 both
     int aeq_occupancy = 0;       // AEQ warps per SM cap (0: as many as resources allow)
-    int aeq_kernel = 0;          // AEQ kernel: 0 auto, 1 a warp per chain, 2 a CTA per chain
-    int cdc_kernel = 0;          // CDC kernel: 0 auto, 1 a block per lane, 2 a block per 8 threads
+    int aeq_kernel = 0;          // AEQ kernel: 0 direct form, 1 a warp per chain, 2 a CTA per chain
+    int cdc_kernel = 0;          // CDC kernel: 0 direct form, 1 a block per lane, 2 a block per 8 threads
     int test_inject = 0;         // DevFrame::flags of the one-shot calls and batches (test hook)
     int smem_per_sm = 0;         // the device's shared memory per SM and per-CTA reserve
     int smem_reserved = 0;
