@@ -507,7 +507,7 @@ def run_fnt(args, rank, world, local_rank, oracle_pool=None):
         e2e["bitexact_vs_device_path"] = bool(torch.equal(oh[0], out_check.cpu()))
         for b_ in rb:
             b_.close()
-        # the one-shot call (fnt_cdc_aeq_run, work lists built per call) on the same buffers
+        # the one-shot call (fnt_cdc_aeq_run) on the same buffers
         fr = [fnt.Frame(xh[0], oh[0], taps, st_e2e)]
         fnt.cdc_aeq_run(plan, fr, host=True)
         t0 = time.perf_counter()
@@ -515,7 +515,7 @@ def run_fnt(args, rank, world, local_rank, oracle_pool=None):
             fnt.cdc_aeq_run(plan, fr, host=True)
         el1 = reduce_max(time.perf_counter() - t0, dev)
         e2e["oneshot"] = {"value": aggregate(n * 5, world, el1), "ms_per_step": el1 / 5 * 1e3,
-                          "api": "fnt_cdc_aeq_run(host_buffers=1), work lists built per call"}
+                          "api": "fnt_cdc_aeq_run(host_buffers=1), one call per step"}
 
     # roofline of the dominant kernel
     aeq_avg = statistics.mean(aeq_ms)
