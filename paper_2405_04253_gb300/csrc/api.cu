@@ -278,8 +278,9 @@ extern "C" fnt_status fnt_plan_set_cdc_kernel(fnt_plan *p, int32_t kind) {
     return FNT_OK;
 }
 
-// One block per lane needs many blocks to fill the GPU; with fewer work items
-// than two per SM, a block per 8 threads (8 warps per item) is taken instead.
+// Of the transform kernels, for a plan that picks neither (the test hook's launches,
+// fnt_plan_cdc_kernel_for): one block per lane needs many blocks to fill the GPU; with
+// fewer work items than two per SM, a block per 8 threads (8 warps per item) does better.
 bool fnt::cdc_use_split(const fnt_plan *p, int64_t n_items) {
     if (p->cdc_kernel != 0) return p->cdc_kernel == 2;
     return n_items < 2 * (int64_t)p->n_sm;
@@ -318,12 +319,13 @@ extern "C" int32_t fnt_plan_aeq_kernel_for(const fnt_plan *p, int64_t n_chains, 
     return aeq_use_serial(p, n_chains, longest_symbols) ? 2 : 1;
 }
 
-// The CTA-per-chain kernel holds one (chain, polarisation) per SM.  It is taken
-// when that many fit in one wave and the longest chain is long enough for its
-// shorter block time to matter (short chains, such as the segments of a
-// served frame, finish sooner in the warp kernel once several launches share
-// the GPU, since each CTA holds a whole SM), and only for per-pair inverse
-// transforms.
+// Of the transform kernels: the CTA-per-chain one holds one (chain, polarisation) per
+// SM.  A plan may pick it; for one that picks none (and runs the direct form),
+// fnt_plan_aeq_kernel_for names it when that many fit in one wave and the longest chain
+// is long enough for its shorter block time to matter (short chains, such as the
+// segments of a served frame, finish sooner in the warp kernel once several launches
+// share the GPU, since each CTA holds a whole SM).  It has per-pair inverse transforms
+// only.
 bool fnt::aeq_use_serial(const fnt_plan *p, int64_t n_chains, int64_t longest_symbols) {
     if (p->d.aeq_freq_sum != 0 || p->aeq_kernel == 1) return false;
     if (p->aeq_kernel == 2) return true;
